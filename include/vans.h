@@ -117,6 +117,15 @@ typedef struct {
  *         only if the cluster holds the domain (D2Q9: at most 2 cells per
  *         thread, D3Q19: 1; two copies of each CTA's rows within 227 KB):
  *         VANS_ERR_UNSUPPORTED otherwise.  Plates on nodes included.
+ * kind 9: `rows` (2..4) steps per launch, D2Q9: each warp walks a strip of
+ *         rows with all the steps as a wave, the populations in between held on
+ *         chip, so that a launch moves the bytes of one step.  cpt 2, warps 4;
+ *         ctas 0..2: strips for that many CTAs per SM (0: as many as fit).  A run
+ *         of n steps is split into launches of equal size or one step apart; a
+ *         single step (vans_step(h, 1), vans_step_raw, the forward steps of
+ *         vans_adjoint_segment, a slab) is a launch of the single-step kind that
+ *         vans_autotune found fastest (kind 0 after vans_set_launch).  Not for
+ *         plates on nodes, nor planes of 4 GB or more (VANS_ERR_UNSUPPORTED).
  * Kinds 1 and 3 are not built (VANS_ERR_ARG).
  *         The batched path takes kinds 0, 2, 4 and 5 (one CTA per strip of
  *         up to 32 rows of one domain) and 6, 7 (one table of every domain's
@@ -128,7 +137,8 @@ typedef struct {
     int kind;
     int ctas;   /* kinds 2-7: at most this many CTAs per SM (1..4; the
                    dynamic shared memory request is raised until no more
-                   fit), 0 = as many as fit; kinds 0 and 8: must be 0 */
+                   fit), 0 = as many as fit; kinds 0 and 8: must be 0;
+                   kind 9: see there */
 } vans_launch;
 
 /* ---------------------------------------------------------------- sizes -- */
@@ -186,6 +196,13 @@ int vans_update_eps(vans_t h, const float *eps_dev);
  * F_i.  Long runs replay a captured CUDA graph.  Errors: VANS_ERR_STATE before
  * vans_set_eps, VANS_ERR_ARG for nsteps < 0, VANS_ERR_CUDA. */
 int vans_step(vans_t h, int nsteps);
+
+/* vans_step by launches of one step each (or the one launch of kind 8), whatever
+ * launch configuration is set: the forward run of a checkpointed reverse pass.
+ * vans_adjoint_segment recomputes its states with the same launches, bit for bit;
+ * those of a run of several steps per launch (kind 9) differ by FP32 roundings.
+ * Errors as vans_step. */
+int vans_step_single(vans_t h, int nsteps);
 
 /* nsteps steps that watch themselves (no extra pass over the populations):
  * the last step of every block of `every` steps (every >= 1; also the last of
@@ -256,8 +273,8 @@ int vans_step_adjoint(vans_t h, const float *state_t, const float *lam_in, float
 
 /* The reverse pass over one checkpointed segment in one call: copies the
  * checkpoint `ckpt` (a state) into seg[0], recomputes len >= 1 forward steps
- * seg[k] -> seg[k+1] with the step kernel (so the states equal the forward
- * run's), then applies len reverse steps from seg[len-1] down to seg[0].  On
+ * seg[k] -> seg[k+1] with the step kernel (so the states equal those of a
+ * forward run of vans_step_single), then applies len reverse steps from seg[len-1] down to seg[0].  On
  * entry lam holds the lambda of seg[len]; on return the lambda of seg[0].  seg
  * is (len+1) state buffers back to back; tmp is a second lambda buffer; the
  * eps partials are added into grad_acc.  The work is captured once per

@@ -97,8 +97,9 @@ class Launch:
     per-warp stage release (5: consecutive cells per thread); kinds 6, 7:
     persistent CTAs over interleaved row tiles; kind 8: every step of a call
     in one launch of one thread-block cluster holding the state in shared
-    memory (rows = the largest cluster, warps 8 or 16, cpt 1).  Kinds 1 and 3
-    are not built.  ctas: at most that many CTAs per SM for the pipelined
+    memory (rows = the largest cluster, warps 8 or 16, cpt 1); kind 9: rows =
+    steps per launch, held on chip (D2Q9, cpt 2, warps 4).  Kinds 1 and 3 are
+    not built.  ctas: at most that many CTAs per SM for the pipelined
     kinds (0: as many as fit)."""
     cpt: int
     warps: int
@@ -137,6 +138,7 @@ def load_library(build_if_missing: bool = True) -> ctypes.CDLL:
             "vans_set_eps_async": (ctypes.c_int, [_H, _F]),
             "vans_update_eps": (ctypes.c_int, [_H, _F]),
             "vans_step": (ctypes.c_int, [_H, ctypes.c_int]),
+            "vans_step_single": (ctypes.c_int, [_H, ctypes.c_int]),
             "vans_step_raw": (ctypes.c_int, [_H, _F, _F]),
             "vans_step_monitored": (ctypes.c_int, [_H, ctypes.c_int, ctypes.c_int, _F, _F, _F]),
             "vans_moments": (ctypes.c_int, [_H, _F, _F]),
@@ -343,6 +345,11 @@ class Solver:
 
     def step(self, nsteps: int = 1):
         _check(self.lib.vans_step(self._h, int(nsteps)), "vans_step")
+
+    def step_single(self, nsteps: int = 1):
+        """``step`` by launches of one step each, whatever launch is set: the
+        forward run whose states ``adjoint_segment`` recomputes bit for bit."""
+        _check(self.lib.vans_step_single(self._h, int(nsteps)), "vans_step_single")
 
     def step_monitored(self, nsteps: int, every: int, rho=None, u=None, stats=None):
         """nsteps steps; every `every` steps the step kernel also writes rho and u

@@ -6,8 +6,8 @@ J = sum over the plane x = x_out of eps*rho*u_x (Eq. 1moment) at the last step,
 keeping a checkpoint of the state every ``every`` steps.  Its backward walks
 the segments newest first: for each, one library call (vans_adjoint_segment,
 a CUDA graph replayed per segment) restores the checkpoint, recomputes the
-segment's states with the same step kernel (so they are bit-identical to the
-forward ones), then applies the hand-written adjoint step kernel to them in
+segment's states with the same step kernel as the forward run, which steps by
+``step_single`` (so they are bit-identical to the forward ones), then applies the hand-written adjoint step kernel to them in
 reverse, accumulating dJ/deps; a final kernel adds the initial condition
 f = w eps and the transposed grad-eps stencil.
 """
@@ -27,7 +27,8 @@ class OutletFlux(torch.autograd.Function):
         while done < nsteps:
             ckpts.append(solver.get_state())
             n = min(every, nsteps - done)
-            solver.step(n)
+            # single-step launches: the segments are recomputed with the same ones
+            solver.step_single(n)
             done += n
         final = solver.get_state()
         J = solver.flux(x_out, state=final)

@@ -90,6 +90,9 @@ bool launch_ok(const vans_launch *c, int q, bool batched) {
     if (c->kind == 8)       // cluster-resident steps: cluster of up to `rows` CTAs
         return !batched && c->cpt == 1 && c->ctas == 0 && (c->warps == 8 || c->warps == 16) &&
                c->rows >= 2 && c->rows <= 16;
+    if (c->kind == 9)       // `rows` steps per launch held in registers
+        return !batched && q == 9 && c->cpt == 2 && c->warps == 4 && c->rows >= 2 &&
+               c->rows <= vans::kMultiMax && c->ctas <= 2;
     // kinds 1 and 3 are not built (never the fastest at any measured size)
     if (c->kind < 2 || c->kind > 7 || c->kind == 3) return false;
     if (c->rows < 2 || c->rows > 6) return false;
@@ -168,7 +171,9 @@ struct vans_s {
     int device = 0;
     long long launches = 0;
     Launch L{4, 4, 1, 0};
-    cudaGraphExec_t gexec[kGraphSizes] = {};   // 64, 32, ..., 2 steps
+    Launch Ls{4, 4, 1, 0};                      // single steps: L, or its stand-in if L is kind 9
+    cudaGraphExec_t gexec[kGraphSizes] = {};   // 64, 32, ..., 2 single-step launches
+    cudaGraphExec_t gmulti[kGraphSizes] = {};  // as many kind 9 launches of L.rows steps
     int *flag = nullptr;                        // device status words (workspace)
     float *mon_part = nullptr;                  // monitoring partial maxima (workspace)
     int adj_fp64 = 0;                           // reverse-step arithmetic in FP64
@@ -208,10 +213,11 @@ namespace {
 int cuda_status(cudaError_t e) { return e == cudaSuccess ? VANS_OK : VANS_ERR_CUDA; }
 
 void drop_graph(vans_t h) {
-    for (auto &g : h->gexec) {
-        if (g) cudaGraphExecDestroy(g);
-        g = nullptr;
-    }
+    for (auto *gs : {h->gexec, h->gmulti})
+        for (int k = 0; k < kGraphSizes; ++k) {
+            if (gs[k]) cudaGraphExecDestroy(gs[k]);
+            gs[k] = nullptr;
+        }
     for (auto &g : h->seg_graphs) cudaGraphExecDestroy(g.exec);
     h->seg_graphs.clear();
 }
@@ -225,20 +231,26 @@ cudaError_t batched_step(vans_t h, cudaStream_t s, int par) {
                                      h->grid, s);
 }
 
-cudaError_t one_step(vans_t h, cudaStream_t s, int par) {
+// the single-step launch of a handle that nobody has tuned
+Launch single_default(int q) { return q == 9 ? Launch{4, 4, 1, 0} : Launch{2, 4, 1, 0}; }
+
+// one launch of `steps` steps (more than one: kind 9)
+cudaError_t one_launch(vans_t h, cudaStream_t s, int par, int steps) {
     ++h->launches;
     if (h->batched) return batched_step(h, s, par);
-    return vans::launch_step(h->q, h->dom, h->st[par], h->st[par ^ 1], h->L, s);
+    if (steps > 1)
+        return vans::launch_multi(h->dom, h->st[par], h->st[par ^ 1], steps, h->L.ctas, s);
+    return vans::launch_step(h->q, h->dom, h->st[par], h->st[par ^ 1], h->Ls, s);
 }
 
-// capture the graph of n steps starting at parity 0
-int capture_steps(vans_t h, int n, cudaGraphExec_t *out) {
+// capture the graph of n launches of `steps` steps starting at parity 0
+int capture_launches(vans_t h, int n, int steps, cudaGraphExec_t *out) {
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return VANS_ERR_CUDA;
     const long long before = h->launches;
     cudaError_t le = cudaSuccess;
-    for (int s = 0; s < n && le == cudaSuccess; ++s) le = one_step(h, h->cap, s & 1);
+    for (int s = 0; s < n && le == cudaSuccess; ++s) le = one_launch(h, h->cap, s & 1, steps);
     h->launches = before;                       // capture does not run anything
     e = cudaStreamEndCapture(h->cap, &g);
     if (le != cudaSuccess || e != cudaSuccess) {
@@ -256,10 +268,10 @@ int capture_steps(vans_t h, int n, cudaGraphExec_t *out) {
 
 // all graph sizes at once, so the first run that needs any of them pays the
 // capture for every later run length
-int ensure_graph(vans_t h) {
-    if (h->gexec[0]) return VANS_OK;
+int ensure_graphs(vans_t h, cudaGraphExec_t *gs, int steps) {
+    if (gs[0]) return VANS_OK;
     for (int k = 0; k < kGraphSizes; ++k) {
-        const int rc = capture_steps(h, kGraphSteps >> k, &h->gexec[k]);
+        const int rc = capture_launches(h, kGraphSteps >> k, steps, &gs[k]);
         if (rc) {
             drop_graph(h);
             return rc;
@@ -268,33 +280,24 @@ int ensure_graph(vans_t h) {
     return VANS_OK;
 }
 
-// nsteps steps; the parity lives in h->cur (single) or h->parity (batched)
-int run_steps(vans_t h, int nsteps) {
+// `count` launches of `steps` steps each, replayed from the graphs gs (nullptr:
+// launched one by one); the parity lives in h->cur (single) or h->parity (batched)
+int run_launches(vans_t h, int count, int steps, cudaGraphExec_t *gs) {
     int &par = h->batched ? h->parity : h->cur;
-    if (!h->batched && h->L.kind == 8 && nsteps > 0) {
-        // all the steps in one launch; the result lands where the step-by-step
-        // run would leave it
-        ++h->launches;
-        if (vans::launch_step_cluster(h->q, h->dom, h->st[par], h->st[par ^ (nsteps & 1)], nsteps,
-                                      h->L, h->stream) != cudaSuccess)
-            return VANS_ERR_CUDA;
-        par ^= nsteps & 1;
-        return VANS_OK;
-    }
-    int left = nsteps;
-    if (left >= 2) {
+    int left = count;
+    if (left >= 2 && gs) {
         if (par != 0) {
-            if (one_step(h, h->stream, par) != cudaSuccess) return VANS_ERR_CUDA;
+            if (one_launch(h, h->stream, par, steps) != cudaSuccess) return VANS_ERR_CUDA;
             par ^= 1;
             --left;
         }
         if (left >= 2) {
-            int rc = ensure_graph(h);
+            int rc = ensure_graphs(h, gs, steps);
             if (rc) return rc;
             for (int k = 0; k < kGraphSizes; ++k) {
                 const int n = kGraphSteps >> k;
                 while (left >= n) {
-                    if (cudaGraphLaunch(h->gexec[k], h->stream) != cudaSuccess) return VANS_ERR_CUDA;
+                    if (cudaGraphLaunch(gs[k], h->stream) != cudaSuccess) return VANS_ERR_CUDA;
                     h->launches += n;
                     left -= n;
                 }
@@ -302,11 +305,39 @@ int run_steps(vans_t h, int nsteps) {
         }
     }
     while (left > 0) {
-        if (one_step(h, h->stream, par) != cudaSuccess) return VANS_ERR_CUDA;
+        if (one_launch(h, h->stream, par, steps) != cudaSuccess) return VANS_ERR_CUDA;
         par ^= 1;
         --left;
     }
     return VANS_OK;
+}
+
+// nsteps steps by single-step launches (kind 8: all of them in one launch)
+int run_single(vans_t h, int nsteps) {
+    if (!h->batched && h->Ls.kind == 8 && nsteps > 0) {
+        // the result lands where the step-by-step run would leave it
+        ++h->launches;
+        if (vans::launch_step_cluster(h->q, h->dom, h->st[h->cur], h->st[h->cur ^ (nsteps & 1)],
+                                      nsteps, h->Ls, h->stream) != cudaSuccess)
+            return VANS_ERR_CUDA;
+        h->cur ^= nsteps & 1;
+        return VANS_OK;
+    }
+    return run_launches(h, nsteps, 1, h->gexec);
+}
+
+// nsteps steps.  Kind 9 takes up to L.rows of them per launch: as few launches as
+// that allows, of equal size or one step apart (9 steps at 4 per launch run as
+// 3 + 3 + 3, not 4 + 4 + 1: a launch of fewer steps saves less than it loses).
+// A single step is a single-step launch.
+int run_steps(vans_t h, int nsteps) {
+    if (h->batched || h->L.kind != 9 || h->slab || nsteps < 2) return run_single(h, nsteps);
+    const int most = h->L.rows, launches = (nsteps + most - 1) / most;
+    const int few = nsteps / launches, longer = nsteps - few * launches;
+    int rc = VANS_OK;
+    if (longer > 0) rc = run_launches(h, longer, few + 1, few + 1 == most ? h->gmulti : nullptr);
+    if (rc) return rc;
+    return run_launches(h, launches - longer, few, few == most ? h->gmulti : nullptr);
 }
 
 int make_streams(vans_t h, void *stream) {
@@ -412,7 +443,7 @@ int set_batch_launch(vans_t h, const Launch &L) {
     return VANS_OK;
 }
 
-// Fastest of three timed trials (after two untimed) of `reps` launches
+// Fastest of three timed trials (after an untimed one) of `reps` launches
 // replayed as one CUDA graph, as run_steps issues them: one noisy trial does
 // not decide the pick, and small domains are not judged by a launch overhead
 // that the graph replay does not pay.  fn(stream) issues one launch; a shape
@@ -437,7 +468,7 @@ float time_launches(vans_t h, F &&fn, int reps) {
     cudaEvent_t a, b;
     cudaEventCreate(&a);
     cudaEventCreate(&b);
-    for (int i = 0; i < 2; ++i) cudaGraphLaunch(ge, h->stream);
+    cudaGraphLaunch(ge, h->stream);
     float best = 1e30f;
     for (int trial = 0; trial < 3; ++trial) {
         cudaEventRecord(a, h->stream);
@@ -496,6 +527,11 @@ std::vector<Launch> candidates(int q, bool batched) {
     }
     // cluster-resident multi-step shapes {1, warps, largest cluster, 8}; the
     // autotuner skips those whose cluster cannot hold the domain
+    if (q == 9)             // kind 9: {2, warps, steps per launch, 9}
+        for (const Launch &m : {Launch{2, 4, 2, 9, 0}, Launch{2, 4, 2, 9, 2}, Launch{2, 4, 3, 9, 0},
+                                Launch{2, 4, 3, 9, 1}, Launch{2, 4, 4, 9, 0}, Launch{2, 4, 4, 9, 1},
+                                Launch{2, 4, 4, 9, 2}})
+            c.push_back(m);
     const Launch k8[] = {{1, 8, 16, 8}, {1, 16, 16, 8}, {1, 8, 8, 8}, {1, 16, 8, 8}};
     c.insert(c.end(), std::begin(k8), std::end(k8));
     return c;
@@ -540,7 +576,7 @@ int vans_create(const vans_params *p, void *workspace, size_t workspace_bytes, v
     h->dom.eps = h->eps_pad;
     h->dom.status = h->flag + 1;
     h->mon_part = (float *)(h->flag + kFlagFloats);
-    h->L = (p->q == 9) ? Launch{4, 4, 1, 0} : Launch{2, 4, 1, 0};
+    h->L = h->Ls = single_default(p->q);
     // the pipelined reverse step, one cell per thread, 4 stages: fastest on GB300 at 512^2
     // (backward pass 17.4 us per step against 20.8 with the register-load kernel)
     h->adjL = (p->q == 19) ? Launch{1, 4, 2, 1} : Launch{1, 4, 4, 1};   // D3Q19: 0.78 vs 0.61 of HBM
@@ -619,6 +655,13 @@ int vans_step(vans_t h, int nsteps) {
     return run_steps(h, nsteps);
 }
 
+int vans_step_single(vans_t h, int nsteps) {
+    if (!h || h->batched || nsteps < 0) return VANS_ERR_ARG;
+    if (!h->eps_set) return VANS_ERR_STATE;
+    if (h->slab && nsteps > 1) return VANS_ERR_UNSUPPORTED;
+    return run_single(h, nsteps);
+}
+
 int vans_step_monitored(vans_t h, int nsteps, int every, float *rho_dev, float *u_dev,
                         float *stats_dev) {
     if (!h || h->batched || nsteps < 0 || every < 1 || !rho_dev || !u_dev || !stats_dev)
@@ -656,7 +699,7 @@ int vans_step_raw(vans_t h, const float *in, float *out) {
     if (!h || h->batched || !in || !out || in == out) return VANS_ERR_ARG;
     if (!h->eps_set) return VANS_ERR_STATE;
     ++h->launches;
-    return cuda_status(vans::launch_step(h->q, h->dom, in, out, h->L, h->stream));
+    return cuda_status(vans::launch_step(h->q, h->dom, in, out, h->Ls, h->stream));
 }
 
 int vans_moments(vans_t h, float *rho_dev, float *u_dev) {
@@ -710,8 +753,10 @@ int vans_set_launch(vans_t h, const vans_launch *cfg) {
     const Launch L{cfg->cpt, cfg->warps, cfg->rows, cfg->kind, cfg->ctas};
     if (!h->batched && h->dom.nee && !vans::launch_has_plates(h->q, L)) return VANS_ERR_UNSUPPORTED;
     if (L.kind == 8 && !vans::cluster_fits(h->q, h->dom, L.rows, L.warps)) return VANS_ERR_UNSUPPORTED;
+    if (L.kind == 9 && !h->slab && !vans::multi_fits(h->q, h->dom)) return VANS_ERR_UNSUPPORTED;
     if (h->batched) return set_batch_launch(h, L);
     h->L = L;
+    h->Ls = L.kind == 9 ? single_default(h->q) : L;
     drop_graph(h);
     return VANS_OK;
 }
@@ -722,32 +767,64 @@ int vans_autotune(vans_t h, vans_launch *chosen) {
     // time each candidate on the current state; the output goes to the other
     // buffer, which holds nothing live, so the state is unchanged
     const std::vector<Launch> cs = candidates(h->q, false);
-    Launch best = h->L;
-    float best_ms = 1e30f;
+    Launch best = h->Ls, single = h->Ls;
+    float best_ms = 1e30f, single_ms = 1e30f;
     const float *in = h->st[h->cur];
     float *outb = h->st[h->cur ^ 1];
     const int reps = h->dom.cells > (1 << 22) ? 5 : 21;
     for (const Launch &L : cs) {
         if (h->dom.nee && !vans::launch_has_plates(h->q, L)) continue;   // no plate instance
         if (L.kind == 8 && !vans::cluster_fits(h->q, h->dom, L.rows, L.warps)) continue;
-        // kind 8 runs the reps steps in one launch (odd reps: the result
-        // lands in the spare buffer, as one step of the other kinds does)
-        const float ms =
-            L.kind == 8
-                ? time_launches(h, [&](cudaStream_t st) {
-                      return vans::launch_step_cluster(h->q, h->dom, in, outb, reps, L, st);
-                  }, 1)
-                : time_launches(h, [&](cudaStream_t st) {
-                      return vans::launch_step(h->q, h->dom, in, outb, L, st);
-                  }, reps);
-        h->launches += L.kind == 8 ? 5 : 5 * reps;
-        if (ms < best_ms) {
-            best_ms = ms;
-            best = L;
+        if (L.kind == 9 && !vans::multi_fits(h->q, h->dom)) continue;
+        // all scored as the time of `reps` steps
+        float ms = 1e30f;
+        if (L.kind == 9) {
+            // several launches in a row, as a run issues them
+            const int n = std::max(2, reps / L.rows);
+            ms = time_launches(h, [&](cudaStream_t st) {
+                return vans::launch_multi(h->dom, in, outb, L.rows, L.ctas, st);
+            }, n) * reps / (float)(n * L.rows);
+            h->launches += 4 * n;
+            if (ms < best_ms) {
+                best_ms = ms;
+                best = L;
+            }
+            continue;
+        }
+        if (L.kind == 8) {
+            // kind 8 runs the steps of a call in one launch: of reps steps, and of
+            // five times as many for the comparison with kind 9 (odd counts: the
+            // result lands in the spare buffer, as one step of the other kinds does)
+            auto steps = [&](int n) {
+                h->launches += 4;
+                return time_launches(h, [&](cudaStream_t st) {
+                    return vans::launch_step_cluster(h->q, h->dom, in, outb, n, L, st);
+                }, 1);
+            };
+            const float many = steps(5 * reps) / 5.f;
+            if (many < best_ms) {
+                best_ms = many;
+                best = L;
+            }
+            ms = steps(reps);
+        } else {
+            ms = time_launches(h, [&](cudaStream_t st) {
+                return vans::launch_step(h->q, h->dom, in, outb, L, st);
+            }, reps);
+            h->launches += 4 * reps;
+            if (ms < best_ms) {
+                best_ms = ms;
+                best = L;
+            }
+        }
+        if (ms < single_ms) {
+            single_ms = ms;
+            single = L;
         }
     }
     if (cudaGetLastError() != cudaSuccess) return VANS_ERR_CUDA;
     h->L = best;
+    h->Ls = best.kind == 9 ? single : best;
     drop_graph(h);
     if (chosen) {
         chosen->cpt = best.cpt;
@@ -819,7 +896,7 @@ int vans_adjoint_segment(vans_t h, const float *ckpt, float *seg, int len, float
         cudaError_t le = cudaSuccess;
         // recompute the segment's states with the forward step kernel
         for (int k = 0; k < len && le == cudaSuccess; ++k)
-            le = vans::launch_step(h->q, h->dom, seg + k * sf, seg + (k + 1) * sf, h->L, h->cap);
+            le = vans::launch_step(h->q, h->dom, seg + k * sf, seg + (k + 1) * sf, h->Ls, h->cap);
         // then walk back through them
         float *a = lam, *b = tmp;
         for (int k = len - 1; k >= 0 && le == cudaSuccess; --k) {
@@ -1107,7 +1184,7 @@ int vans_batch_autotune(vans_t h, vans_launch *chosen) {
         // reads the current parity and writes the other buffer of every domain
         const float ms =
             time_launches(h, [&](cudaStream_t st) { return batched_step(h, st, par); }, 5);
-        h->launches += 25;
+        h->launches += 20;
         if (ms < best_ms) {
             best_ms = ms;
             best = L;

@@ -55,6 +55,7 @@ struct Tile {
 //         thread per tile, rows = pipeline stages)
 // kind 8: cluster-resident multi-step kernel (32*warps threads per CTA, rows =
 //         the largest cluster)
+// kind 9: rows (2..kMultiMax) steps per launch, held on chip (D2Q9)
 // ctas: at most that many CTAs per SM for the pipelined kinds (0: as many as fit)
 struct Launch {
     int cpt, warps, rows, kind;
@@ -89,6 +90,14 @@ cudaError_t launch_step_tma(int q, const VDom &d, const float *fin, float *fout,
 // whole state in its shared memory; reads fin, writes fout (which may be fin)
 cudaError_t launch_step_cluster(int q, const VDom &d, const float *fin, float *fout, int nsteps,
                                 Launch L, cudaStream_t stream);
+// kind 9 (D2Q9, x periodic within the domain, no plates on nodes): `steps`
+// (2..kMultiMax) steps in one launch, in strips for `ctas` CTAs per SM (0: chosen)
+constexpr int kMultiMax = 4;
+// whether kind 9 takes the domain: D2Q9, no plates on nodes, not a slab, planes
+// of less than 4 GB
+bool multi_fits(int q, const VDom &d);
+cudaError_t launch_multi(const VDom &d, const float *fin, float *fout, int steps, int ctas,
+                         cudaStream_t stream);
 // whether a cluster of at most cmax CTAs of `warps` warps holds the domain
 // (never plates on nodes)
 bool cluster_fits(int q, const VDom &d, int cmax, int warps);

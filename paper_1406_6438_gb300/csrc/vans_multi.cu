@@ -1,0 +1,592 @@
+// vans_multi.cu -- two to four time steps per launch with the steps in between
+// held on chip (launch kind 9, D2Q9).
+//
+// One step of the other kinds reads and writes every population: 76 bytes per
+// cell update, which is what bounds them (4096^2: 197 us per step, 0.95 of the copy
+// bandwidth).  Here a warp walks down a strip of rows of one 64-column block, two
+// adjacent cells per lane, and carries T steps along as a wave: when it has loaded
+// row r it computes step 1 of row r, step 2 of row r-1, ..., step T of row r-T+1,
+// and stores only the last.  What step l+1 of a row still needs of step l's rows
+// stays with the lane (the +-1 column shift of the pull is a shuffle), so a launch
+// moves 76 bytes per cell for T steps.  No barrier, no shared state between warps:
+// the outer ghost_cols columns of a block are computed redundantly (8 of 64 for
+// T = 3, 4), as are the T-1 rows before and after a strip.
+//
+// What bounds it is the FP32 pipe and its latency: an update of a pair of cells is
+// 91 packed instructions (fma.rn.f32x2 takes the pipe for two cycles, three with
+// three register operands, but one issue slot), 220 cycles per warp at four warps
+// per scheduler, 350 for a lone one.  Hence what does not change from step to step
+// (the porosity terms, 13 pairs per cell) is formed once per row and kept in
+// shared memory, the e_y > 0 values that wait two turns are kept there too (in
+// registers they cost 12 per step and as many moves), and the next row's loads go
+// out before the last step: 160-168 registers, 12 warps per SM, none spilled.
+// Measured at 4096^2 (us per step; ncu: DRAM 0.3 of its peak): T = 2 135, 3 107,
+// 4 101, periodic or between walls; 2048^2 27, 1024^2 8.4 (kind 7: 12.2), 512^2
+// 3.8 (kind 0: 4.9).  With 128 registers (16 warps) T = 2 gains 3 %, 3 and 4
+// spill and lose.
+//
+// Every operation is written out as a rounded multiply-add, addition or
+// multiplication, so that nothing is left to the compiler's contraction: the
+// result does not depend on T, on the strips or on the column blocks.
+#include "vans_device.cuh"
+
+namespace vans {
+
+namespace {
+
+using f2 = float2;
+
+__device__ __forceinline__ f2 bc(float v) { return make_float2(v, v); }
+__device__ __forceinline__ f2 add2(f2 a, f2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ f2 sub2(f2 a, f2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
+__device__ __forceinline__ f2 neg2(f2 a) { return make_float2(-a.x, -a.y); }
+
+__device__ __forceinline__ float rcp_ftz(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float rsqrt_ftz(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// the hardware estimates with one Newton-Raphson step each, as rcp_nr and
+// sqrt_nr (vans_device.cuh); sqrt2 takes x > 0, normal
+__device__ __forceinline__ f2 rcp2(f2 x) {
+    const f2 r = make_float2(rcp_ftz(x.x), rcp_ftz(x.y));
+    return fma2(r, fma2(neg2(x), r, bc(1.f)), r);
+}
+__device__ __forceinline__ f2 sqrt2(f2 x) {
+    const f2 y = make_float2(rsqrt_ftz(x.x), rsqrt_ftz(x.y));
+    const f2 s = mul2(x, y);
+    return fma2(mul2(y, bc(0.5f)), fma2(neg2(s), s, x), s);
+}
+
+// What a cell's update needs of the porosity, formed once per row and launch:
+// eps, Hc = cs^2 grad eps / eps + g, the drag coefficients and w_i (eps - eps~_i).
+// Fourteen pairs (one spare), seven 16-byte words per lane.
+struct Por {
+    f2 e0, hx, hy, al, be;
+    f2 wd[9];              // wd[0] unused
+};
+
+// pair of cells (x, x+1) with the neighbours on either side: values at x-1 .. x+2
+struct Row {
+    float l;
+    f2 c;
+    float r;
+    __device__ f2 left() const { return make_float2(l, c.x); }
+    __device__ f2 right() const { return make_float2(c.y, r); }
+};
+
+__device__ __forceinline__ Row with_neighbours(f2 c) {
+    Row o;
+    o.c = c;
+    o.l = __shfl_up_sync(VANS_FULL, c.y, 1);
+    o.r = __shfl_down_sync(VANS_FULL, c.x, 1);
+    return o;
+}
+
+// values one column to the left (s < 0: what a population moving +x pulls) or
+// right of each cell of the pair
+__device__ __forceinline__ f2 from_left(f2 c) {
+    return make_float2(__shfl_up_sync(VANS_FULL, c.y, 1), c.x);
+}
+__device__ __forceinline__ f2 from_right(f2 c) {
+    return make_float2(c.y, __shfl_down_sync(VANS_FULL, c.x, 1));
+}
+
+// direction order: 0 (0,0), 1 (1,0), 2 (0,1), 3 (-1,0), 4 (0,-1), 5 (1,1),
+// 6 (-1,1), 7 (-1,-1), 8 (1,-1); m, z, p: the porosity rows y-1, y, y+1
+__device__ __forceinline__ void porosity_terms(const VDom &d, const Row &m, const Row &z, const Row &p,
+                                               bool lo_wall, bool hi_wall, Por &o) {
+    const f2 e0 = z.c;
+    f2 et[9];
+    et[1] = z.right();
+    et[3] = z.left();
+    et[2] = p.c;
+    et[5] = p.right();
+    et[6] = p.left();
+    et[4] = m.c;
+    et[8] = m.right();
+    et[7] = m.left();
+    if (hi_wall) et[2] = et[5] = et[6] = e0;     // past a wall: eps(x)
+    if (lo_wall) et[4] = et[7] = et[8] = e0;
+    const f2 d1 = sub2(et[1], et[3]), d2 = sub2(et[2], et[4]);
+    const f2 d5 = sub2(et[5], et[7]), d8 = sub2(et[8], et[6]);
+    // grad eps = (4 d1 + d5 + d8, 4 d2 + d5 - d8) / 12
+    const f2 gx = fma2(d1, bc(4.f), add2(d5, d8)), gy = fma2(d2, bc(4.f), sub2(d5, d8));
+    const f2 inv = make_float2(rcp_nr(e0.x), rcp_nr(e0.y));
+    const f2 inv36 = mul2(inv, bc(1.f / 36.f));
+    o.e0 = e0;
+    o.hx = fma2(gx, inv36, bc(d.g[0]));
+    o.hy = fma2(gy, inv36, bc(d.g[1]));
+    // the drag law (drag of vans_device.cuh) for the pair
+    if (d.k_mode == 0) {
+        const f2 om = sub2(bc(1.f), e0);
+        o.al = mul2(mul2(mul2(om, bc(d.ca)), om), inv);
+        o.be = mul2(om, bc(d.cb));
+    } else {
+        const f2 ee = mul2(e0, e0);
+        o.al = mul2(ee, bc(d.ca));
+        o.be = mul2(d.k_mode == 1 ? mul2(ee, e0)
+                                  : mul2(e0, sqrt2(make_float2(fmaxf(e0.x, 1e-36f), fmaxf(e0.y, 1e-36f)))),
+                    bc(d.cb));
+    }
+    if (d.drag_mode == 0) o.al = bc(0.f);
+    if (d.drag_mode != 2) o.be = bc(0.f);
+#pragma unroll
+    for (int i = 1; i < 9; ++i) o.wd[i] = mul2(sub2(e0, et[i]), bc(Lat<9>::w(i)));
+}
+
+// One update of a pair of cells: the final LBE in deviation form (macro and
+// collide of vans_device.cuh), with M = 2m, so that u = M / D, and
+// t = p grad eps + R g = R Hc.  With q = omega R u + ct V the odd part of
+// f^eq + P_i + F_i is 3 e.q and, with g = q - omega R u / 2, the even part
+// 9 (e.u)(e.g) - 3 u.g.  The momentum a cell gains is (1 - omega) j + q = j + V
+// only if ct + omega/2 = 1: near rest j = -V/2 is large (the pressure term
+// p grad eps, which the lattice takes back), so a rounding of 3e-8 in that sum
+// is a spurious force; ct is therefore 1 - omega/2, exact in FP32, and both
+// constants enter unscaled (scaled by 3 and rounded again, the velocity was 2 to
+// 3 times further from 64 bits at tau = 0.55 .. 0.6).
+__device__ __forceinline__ void collide_pair(const VDom &d, const f2 h[9], const Por &P, f2 o[9]) {
+    const f2 dl = add2(add2(add2(add2(h[1], h[3]), add2(h[2], h[4])),
+                            add2(add2(h[5], h[7]), add2(h[6], h[8]))), h[0]);
+    const f2 R = add2(P.e0, dl);
+    const f2 d1 = sub2(h[1], h[3]), d2 = sub2(h[2], h[4]);
+    const f2 d5 = sub2(h[5], h[7]), d8 = sub2(h[8], h[6]);
+    const f2 jx = add2(d1, add2(d5, d8)), jy = add2(d2, sub2(d5, d8));
+    const f2 tx = mul2(R, P.hx), ty = mul2(R, P.hy);
+    const f2 Mx = fma2(bc(2.f), jx, tx), My = fma2(bc(2.f), jy, ty);
+    const f2 m2 = fma2(Mx, Mx, mul2(My, My));
+    // |M|; the floor keeps the root finite at rest and is far below any effect
+    const f2 M = sqrt2(make_float2(fmaxf(m2.x, 1e-36f), fmaxf(m2.y, 1e-36f)));
+    const f2 a = fma2(bc(0.5f), P.al, R);
+    const f2 s = rcp2(add2(a, sqrt2(fma2(P.be, M, mul2(a, a)))));
+    const f2 ux = mul2(Mx, s), uy = mul2(My, s);
+    const f2 kd = neg2(fma2(P.be, mul2(M, s), P.al));
+    const f2 Vx = fma2(kd, ux, tx), Vy = fma2(kd, uy, ty);
+    const float om = d.omega;
+    const f2 ct = bc(1.f - 0.5f * om), om1 = bc(1.f - om);
+    const f2 omR = mul2(R, bc(om)), hR = mul2(omR, bc(-0.5f));
+    const f2 qx = fma2(omR, ux, mul2(ct, Vx)), qy = fma2(omR, uy, mul2(ct, Vy));
+    const f2 gx = fma2(hR, ux, qx), gy = fma2(hR, uy, qy);
+    const f2 xx = mul2(ux, gx), yy = mul2(uy, gy), xy = fma2(ux, gy, mul2(uy, gx));
+    const f2 ug = add2(xx, yy);
+    const f2 c = fma2(bc(-3.f), ug, mul2(bc(om), dl));
+    o[0] = fma2(om1, h[0], mul2(bc(Lat<9>::w(0)), c));
+    auto pair = [&](int i, int j, f2 even, f2 q) {
+        const f2 w = bc(Lat<9>::w(i));
+        o[i] = fma2(w, fma2(bc(3.f), q, even), fma2(om1, h[i], P.wd[i]));
+        o[j] = fma2(w, fma2(bc(-3.f), q, even), fma2(om1, h[j], P.wd[j]));
+    };
+    pair(1, 3, fma2(bc(9.f), xx, c), qx);
+    pair(2, 4, fma2(bc(9.f), yy, c), qy);
+    const f2 b = fma2(bc(9.f), ug, c);
+    pair(5, 7, fma2(bc(9.f), xy, b), add2(qx, qy));
+    pair(8, 6, fma2(bc(-9.f), xy, b), sub2(qx, qy));
+}
+
+constexpr int kMultiWarps = 4;      // warps per block, each on its own
+constexpr int kPorBytes = 13 * 8 * 32;   // Por of one warp and row
+
+// columns on each side of a block that are computed but not stored: one per
+// step, even so that the pairs stay aligned
+__host__ __device__ constexpr int ghost_cols(int T) { return (T + 1) & ~1; }
+__host__ __device__ constexpr int out_cols(int T) { return 64 - 2 * ghost_cols(T); }
+
+__device__ __forceinline__ void por_put(float4 *slot, int lane, const Por &P) {
+    slot[0 * 32] = make_float4(P.e0.x, P.e0.y, P.hx.x, P.hx.y);
+    slot[1 * 32] = make_float4(P.hy.x, P.hy.y, P.al.x, P.al.y);
+    slot[2 * 32] = make_float4(P.be.x, P.be.y, P.wd[1].x, P.wd[1].y);
+    slot[3 * 32] = make_float4(P.wd[2].x, P.wd[2].y, P.wd[3].x, P.wd[3].y);
+    slot[4 * 32] = make_float4(P.wd[4].x, P.wd[4].y, P.wd[5].x, P.wd[5].y);
+    slot[5 * 32] = make_float4(P.wd[6].x, P.wd[6].y, P.wd[7].x, P.wd[7].y);
+    reinterpret_cast<f2 *>(slot - lane + 6 * 32)[lane] = P.wd[8];
+}
+
+__device__ __forceinline__ void por_get(const float4 *slot, int lane, Por &P) {
+    float4 t = slot[0 * 32];
+    P.e0 = make_float2(t.x, t.y); P.hx = make_float2(t.z, t.w);
+    t = slot[1 * 32];
+    P.hy = make_float2(t.x, t.y); P.al = make_float2(t.z, t.w);
+    t = slot[2 * 32];
+    P.be = make_float2(t.x, t.y); P.wd[1] = make_float2(t.z, t.w);
+    t = slot[3 * 32];
+    P.wd[2] = make_float2(t.x, t.y); P.wd[3] = make_float2(t.z, t.w);
+    t = slot[4 * 32];
+    P.wd[4] = make_float2(t.x, t.y); P.wd[5] = make_float2(t.z, t.w);
+    t = slot[5 * 32];
+    P.wd[6] = make_float2(t.x, t.y); P.wd[7] = make_float2(t.z, t.w);
+    P.wd[8] = reinterpret_cast<const f2 *>(slot - lane + 6 * 32)[lane];
+}
+
+__device__ __forceinline__ int wrap(int c, int n) {
+    while (c < 0) c += n;
+    while (c >= n) c -= n;
+    return c;
+}
+
+// One warp's strip of rows [y0, y1) of a 64-column block.  WALLS: bounce-back
+// walls on the y faces.  The wave runs through the rows past a wall as well (they
+// wrap around like a periodic axis's and nothing of them is kept); what a row
+// next to a wall pulls from there is put in its place first: the entry that
+// bounced off, at the column from which the shift brings it home.
+template <int T, bool WALLS>
+struct Strip {
+    static constexpr int GL = ghost_cols(T);
+    const VDom &d;
+    const float *__restrict__ fin;
+    float *__restrict__ fout;
+    unsigned char *ring;           // this warp's T rows of Por words
+    f2 *up;                        // this lane's part of the kept e_y > 0 values
+    int x, ia, y0, y1, lane, r, slot, odd;
+    int yp;                        // the row at op
+    uint32_t second;               // bytes from the lane's first column to its second
+    uint32_t om, oz, op, out;      // byte offsets of the rows below, at and above the
+                                   // next row to load, and of the next row to store
+    bool inside, xedge;
+    Row em, ez;                    // porosity rows r-1, r
+    f2 raw[9], enext;              // row r of step 1 and porosity row r+1, loaded a turn ahead
+    // per step l = 1 .. T-1: what step l+1 still needs of earlier rows, shifted:
+    // the e_y = 0 values of one row back in registers, the e_y > 0 values of two
+    // rows back in shared memory, [l][turn parity][direction]
+    f2 mid[T - 1][3];
+
+    // pair of plane p at byte offset `off` of this lane's first column
+    __device__ __forceinline__ f2 load(const float *p, uint32_t off) const {
+        const char *q = reinterpret_cast<const char *>(p);
+        return inside ? __ldg(reinterpret_cast<const f2 *>(q + off))
+                      : make_float2(__ldg(reinterpret_cast<const float *>(q + off)),
+                                    __ldg(reinterpret_cast<const float *>(q + (uint32_t)(off + second))));
+    }
+    // the pair s columns to the right (s = -1, 1) in row y
+    __device__ __forceinline__ f2 load_beside(const float *p, int y, int s) const {
+        const float *row = p + (long long)y * d.pitch + d.off;
+        return make_float2(__ldg(row + wrap(x + s, d.nx)), __ldg(row + wrap(x + 1 + s, d.nx)));
+    }
+    __device__ __forceinline__ float4 *por_row(int k) const {
+        return reinterpret_cast<float4 *>(ring + k * kPorBytes) + lane;
+    }
+    __device__ __forceinline__ f2 *up_row(int l, int par) const {
+        return up + ((l - 1) * 2 + par) * (3 * 32);
+    }
+    __device__ __forceinline__ uint32_t row_off(int y) const {       // 0 <= y < ny
+        return ((uint32_t)y * (uint32_t)d.pitch + (uint32_t)(d.off + ia)) * 4u;
+    }
+    // the populations that step 1 of row y (at offset oz; rows om, op below and
+    // above it) pulls, not yet shifted in x, and the porosity row above
+    template <bool W>
+    __device__ __forceinline__ void load_row(int y) {
+        const long long plane = d.plane;
+        enext = load(d.eps, op);
+        raw[0] = load(fin, oz);
+        raw[1] = load(fin + 1 * plane, oz);
+        raw[3] = load(fin + 3 * plane, oz);
+        raw[2] = load(fin + 2 * plane, om);
+        raw[5] = load(fin + 5 * plane, om);
+        raw[6] = load(fin + 6 * plane, om);
+        raw[4] = load(fin + 4 * plane, op);
+        raw[7] = load(fin + 7 * plane, op);
+        raw[8] = load(fin + 8 * plane, op);
+        if (W && y == 0) {
+            raw[2] = load(fin + 4 * plane, oz);
+            raw[5] = load_beside(fin + 7 * plane, y, 1);
+            raw[6] = load_beside(fin + 8 * plane, y, -1);
+        }
+        if (W && y == d.ny - 1) {
+            raw[4] = load(fin + 2 * plane, oz);
+            raw[7] = load_beside(fin + 5 * plane, y, -1);
+            raw[8] = load_beside(fin + 6 * plane, y, 1);
+        }
+    }
+    template <bool W>
+    __device__ __forceinline__ void prefetch() {                     // row r + 1
+        om = oz;
+        oz = op;
+        if (++yp == d.ny) yp = 0;
+        op = row_off(yp);
+        load_row<W>(r + 1);
+    }
+    __device__ __forceinline__ void moving_wall(const Por &P, f2 h[9]) const {
+        h[4] = fma2(P.e0, bc(wall_gain<9>(d, 4, 1.f)), h[4]);
+        h[7] = fma2(P.e0, bc(wall_gain<9>(d, 7, 1.f)), h[7]);
+        h[8] = fma2(P.e0, bc(wall_gain<9>(d, 8, 1.f)), h[8]);
+    }
+    // step 1 of row r
+    template <bool W>
+    __device__ __forceinline__ void first(f2 o[9]) {
+        const Row ep = with_neighbours(enext);
+        f2 h[9];
+        h[0] = raw[0];
+        h[1] = from_left(raw[1]);
+        h[3] = from_right(raw[3]);
+        h[2] = raw[2];
+        h[5] = from_left(raw[5]);
+        h[6] = from_right(raw[6]);
+        h[4] = raw[4];
+        h[7] = from_right(raw[7]);
+        h[8] = from_left(raw[8]);
+        Por P;
+        const bool above = W && r == d.ny - 1;
+        porosity_terms(d, em, ez, ep, W && r == 0, above, P);
+        por_put(por_row(slot), lane, P);
+        em = ez;
+        ez = ep;
+        if (above && d.moving) moving_wall(P, h);
+        collide_pair(d, h, P, o);
+    }
+    // step l+1 of the row before the one whose step-l values are o
+    template <bool W>
+    __device__ __forceinline__ void next(int l, const f2 o[9], f2 on[9]) {
+        Por P;
+        const int back = slot - l < 0 ? slot - l + T : slot - l;
+        por_get(por_row(back), lane, P);
+        f2 h[9];
+        h[0] = mid[l - 1][0];
+        h[1] = mid[l - 1][1];
+        h[3] = mid[l - 1][2];
+        const f2 *u = up_row(l, odd);                  // written two turns ago
+        h[2] = u[0 * 32];
+        h[5] = u[1 * 32];
+        h[6] = u[2 * 32];
+        h[4] = o[4];
+        h[7] = from_right(o[7]);
+        h[8] = from_left(o[8]);
+        if (W && d.moving && r - l == d.ny - 1) moving_wall(P, h);
+        collide_pair(d, h, P, on);
+    }
+    // what step l+1 needs later of step l's row o (shifted only now: shifted before
+    // next() ran, the new values would need registers beside the old ones)
+    __device__ __forceinline__ void keep(int l, const f2 o[9]) {
+        f2 *u = up_row(l, odd);
+        u[0 * 32] = o[2];
+        u[1 * 32] = from_left(o[5]);
+        u[2 * 32] = from_right(o[6]);
+        mid[l - 1][0] = o[0];
+        mid[l - 1][1] = from_left(o[1]);
+        mid[l - 1][2] = from_right(o[3]);
+    }
+    // step T's row y
+    __device__ __forceinline__ void store(const f2 o[9]) {
+        const long long plane = d.plane;
+        char *q = reinterpret_cast<char *>(fout) + out;
+        out += (uint32_t)d.pitch * 4u;
+        if (!xedge) {
+            if (lane >= GL / 2 && lane < 32 - GL / 2) {
+#pragma unroll
+                for (int i = 0; i < 9; ++i) *reinterpret_cast<f2 *>(q + i * plane * 4) = o[i];
+            }
+            return;
+        }
+        if (lane < GL / 2 || lane >= 32 - GL / 2 || x >= d.nx) return;
+        float *row = reinterpret_cast<float *>(q);
+        const bool both = x + 1 < d.nx;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            row[i * plane] = o[i].x;
+            if (both) row[i * plane + 1] = o[i].y;
+        }
+        if (x == 0) {                                  // column nx mirrors column 0 (e_x < 0)
+            row[3 * plane + d.nx] = o[3].x;
+            row[6 * plane + d.nx] = o[6].x;
+            row[7 * plane + d.nx] = o[7].x;
+        }
+        if (x + 2 >= d.nx) {                           // column -1 mirrors column nx-1 (e_x > 0)
+            float *left = row - x - 1;
+            left[1 * plane] = both ? o[1].y : o[1].x;
+            left[5 * plane] = both ? o[5].y : o[5].x;
+            left[8 * plane] = both ? o[8].y : o[8].x;
+        }
+    }
+    // one turn with steps 1 .. N running (N < T while the wave starts up).  W: a
+    // step's row of this turn, or the row loaded for the next, may lie next to a
+    // wall or just past one
+    template <int N, bool W>
+    __device__ __forceinline__ void turn(bool more) {
+        f2 o[9];
+        first<W>(o);
+#pragma unroll
+        for (int l = 1; l < T; ++l) {
+            if (l > N) break;
+            // the next turn's row, before the last step: earlier, the twenty
+            // registers it lands in would be live through every step
+            if (l == T - 1 && more) prefetch<W>();
+            if (W && r - l + 1 == d.ny) {  // past the upper wall: row ny-1 bounced
+                const f2 *u = up_row(l, odd ^ 1);
+                o[4] = u[0 * 32];
+                o[7] = u[1 * 32];
+                o[8] = u[2 * 32];
+            }
+            f2 on[9];
+            if (l < N) next<W>(l, o, on);
+            keep(l, o);
+            if (W && r - l + 1 == 0) {     // below the lower wall: row 0 bounced
+                f2 *u = up_row(l, odd ^ 1);
+                u[0 * 32] = o[4];
+                u[1 * 32] = o[7];
+                u[2 * 32] = o[8];
+            }
+            if (l < N) {
+#pragma unroll
+                for (int i = 0; i < 9; ++i) o[i] = on[i];
+            }
+        }
+        if (N < T - 1 && more) prefetch<W>();
+        if (N == T) store(o);
+        ++r;
+        odd ^= 1;
+        if (++slot == T) slot = 0;
+    }
+    // step l+1 starts two turns after step l: its first row is one further on, and
+    // the row before it takes one more
+    template <int N>
+    __device__ __forceinline__ void start() {
+        if constexpr (N < T) {
+#pragma unroll 1
+            for (int k = 0; k < 2; ++k) turn<N, WALLS>(true);
+            start<N + 1>();
+        }
+    }
+    __device__ __forceinline__ void run(int xs) {
+        x = xs - GL + 2 * lane;                        // the lane's first column
+        inside = xs - GL >= 0 && xs - GL + 64 <= d.nx;
+        xedge = xs == 0 || xs + out_cols(T) >= d.nx;
+        ia = inside ? x : wrap(x, d.nx);
+        second = inside ? 4u : (uint32_t)(wrap(x + 1, d.nx) - ia) * 4u;
+        slot = 0;
+        odd = 0;
+        r = y0 - (T - 1);
+        out = ((uint32_t)y0 * (uint32_t)d.pitch + (uint32_t)(d.off + x)) * 4u;
+        om = row_off(wrap(r - 1, d.ny));
+        oz = row_off(wrap(r, d.ny));
+        yp = wrap(r + 1, d.ny);
+        op = row_off(yp);
+        em = with_neighbours(load(d.eps, om));
+        ez = with_neighbours(load(d.eps, oz));
+        load_row<WALLS>(r);
+#pragma unroll
+        for (int l = 1; l < T; ++l)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                mid[l - 1][k] = bc(0.f);
+                up_row(l, 0)[k * 32] = up_row(l, 1)[k * 32] = bc(0.f);
+            }
+        const int last = y1 - 1 + (T - 1);             // row of step 1 in the last turn
+        start<1>();
+        if constexpr (!WALLS) {
+#pragma unroll 1
+            while (r <= last) turn<T, false>(r < last);
+        } else {
+            // near the lower wall, away from walls, near the upper one (a turn also
+            // loads row r + 1): one copy of the wall's turn, so that the registers
+            // of the plain one are left alone
+            int until = min(last, T - 1);
+#pragma unroll 1
+            for (;;) {
+#pragma unroll 1
+                while (r <= until) turn<T, true>(r < last);
+                if (r > last) break;
+#pragma unroll 1
+                while (r <= min(last, d.ny - 3)) turn<T, false>(r < last);
+                until = last;
+            }
+        }
+    }
+};
+
+// shared memory of one warp: T rows of Por, two turns of three pairs for each
+// step but the last
+template <int T>
+__host__ __device__ constexpr int warp_smem() {
+    return T * kPorBytes + (T - 1) * 2 * 3 * 8 * 32;
+}
+
+// Unit (strip, column block) of this warp.
+template <int T, bool WALLS>
+__global__ void __launch_bounds__(32 * kMultiWarps, 3)
+    k_multi(const VDom d, const float *__restrict__ fin, float *__restrict__ fout, int ncol,
+            int nstrip) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int unit = blockIdx.x * kMultiWarps + warp;
+    if (unit >= ncol * nstrip) return;
+    const int strip = unit / ncol, col = unit - strip * ncol;
+    unsigned char *ring = smem + warp * warp_smem<T>();
+    f2 *up = reinterpret_cast<f2 *>(ring + T * kPorBytes) + lane;
+    Strip<T, WALLS> s{d, fin, fout, ring, up};
+    s.y0 = (int)((long long)strip * d.ny / nstrip);
+    s.y1 = (int)((long long)(strip + 1) * d.ny / nstrip);
+    s.lane = lane;
+    s.run(col * out_cols(T));
+}
+
+template <int T, bool WALLS>
+cudaError_t launch_multi_t(const VDom &d, const float *fin, float *fout, int ctas,
+                           cudaStream_t stream) {
+    auto kern = k_multi<T, WALLS>;
+    const size_t smem = (size_t)kMultiWarps * warp_smem<T>();
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    int dev = 0, sms = 0, occ = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 32 * kMultiWarps, smem);
+    if (e != cudaSuccess) return e;
+    if (occ < 1) return cudaErrorInvalidConfiguration;
+    const int ncol = (d.nx + out_cols(T) - 1) / out_cols(T);
+    // Strips per column block: the count with the smallest waves x turns (a strip
+    // of n rows takes n + 2 (T-1) turns, and its start is worth one more), a wave
+    // being as many warps as the chip holds, or ctas blocks per SM in one wave:
+    // fewer and longer strips repeat fewer rows, which is the better choice where
+    // short strips would be half repetition (1024^2, T = 4: 9.0 us per step with
+    // 3 blocks per SM, 8.4 with 1)
+    const long long resident = (long long)sms * (ctas > 0 && ctas < occ ? ctas : occ) * kMultiWarps;
+    int nstrip = 1;
+    double best = 1e300;
+    for (int s = 1; s <= d.ny; ++s) {
+        const long long units = (long long)ncol * s;
+        const long long waves = (units + resident - 1) / resident;
+        const double cost = (double)waves * ((d.ny + s - 1) / s + 2 * (T - 1) + 1);
+        if (cost < best) {
+            best = cost;
+            nstrip = s;
+        }
+        if (units > (ctas > 0 ? 1 : 8) * resident) break;
+    }
+    const long long grid = ((long long)ncol * nstrip + kMultiWarps - 1) / kMultiWarps;
+    if (grid > 0x7fffffffLL / kMultiWarps) return cudaErrorInvalidConfiguration;
+    kern<<<(unsigned)grid, 32 * kMultiWarps, smem, stream>>>(d, fin, fout, ncol, nstrip);
+    return cudaGetLastError();
+}
+
+template <int T>
+cudaError_t launch_steps(const VDom &d, const float *fin, float *fout, int ctas,
+                         cudaStream_t stream) {
+    return d.wall_y ? launch_multi_t<T, true>(d, fin, fout, ctas, stream)
+                    : launch_multi_t<T, false>(d, fin, fout, ctas, stream);
+}
+
+}  // namespace
+
+bool multi_fits(int q, const VDom &d) {
+    // byte offsets within a plane are 32-bit
+    return q == 9 && !d.nee && d.xwrap && d.plane < (1LL << 30);
+}
+
+cudaError_t launch_multi(const VDom &d, const float *fin, float *fout, int steps, int ctas,
+                         cudaStream_t stream) {
+    if (!multi_fits(9, d)) return cudaErrorInvalidValue;
+    switch (steps) {
+        case 2: return launch_steps<2>(d, fin, fout, ctas, stream);
+        case 3: return launch_steps<3>(d, fin, fout, ctas, stream);
+        case 4: return launch_steps<4>(d, fin, fout, ctas, stream);
+    }
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace vans
