@@ -126,10 +126,11 @@ typedef struct {
  *         vans_adjoint_segment, a slab) is a launch of the single-step kind that
  *         vans_autotune found fastest (kind 0 after vans_set_launch).  Not for
  *         plates on nodes, nor planes of 4 GB or more (VANS_ERR_UNSUPPORTED).
+ *         In a batch ctas chooses the rows of a strip (0: 96, 1: 48, 2: 192).
  * Kinds 1 and 3 are not built (VANS_ERR_ARG).
  *         The batched path takes kinds 0, 2, 4 and 5 (one CTA per strip of
- *         up to 32 rows of one domain) and 6, 7 (one table of every domain's
- *         row tiles); the batch is D2Q9 only. */
+ *         up to 32 rows of one domain), 6, 7 (one table of every domain's
+ *         row tiles) and 9; the batch is D2Q9 only. */
 typedef struct {
     int cpt;
     int warps;
@@ -326,7 +327,8 @@ int vans_batch_autotune(vans_t h, vans_launch *chosen);
  * *n_records, the number of CTA slots a step can use, is set (the capacity
  * must be 3 * *n_records).  The caller derives the load balance, e.g. the
  * mean over SMs of their busy span over the step's makespan.  The pipelined
- * kinds only (2, 4-7): VANS_ERR_UNSUPPORTED for kind 0. */
+ * kinds only (2, 4-7; kind 9: its single-step launch): VANS_ERR_UNSUPPORTED for
+ * kind 0. */
 int vans_batch_profile_step(vans_t h, unsigned long long *records_dev, long long capacity,
                             long long *n_records);
 /* Cells summed over all domains. */

@@ -91,7 +91,7 @@ bool launch_ok(const vans_launch *c, int q, bool batched) {
         return !batched && c->cpt == 1 && c->ctas == 0 && (c->warps == 8 || c->warps == 16) &&
                c->rows >= 2 && c->rows <= 16;
     if (c->kind == 9)       // `rows` steps per launch held in registers
-        return !batched && q == 9 && c->cpt == 2 && c->warps == 4 && c->rows >= 2 &&
+        return q == 9 && c->cpt == 2 && c->warps == vans::kMultiWarps && c->rows >= 2 &&
                c->rows <= vans::kMultiMax && c->ctas <= 2;
     // kinds 1 and 3 are not built (never the fastest at any measured size)
     if (c->kind < 2 || c->kind > 7 || c->kind == 3) return false;
@@ -194,7 +194,10 @@ struct vans_s {
     VDom *doms_d = nullptr;
     Tile *tiles_d = nullptr;
     long long tile_cap = 0;
-    std::vector<Tile> tiles;
+    std::vector<Tile> tiles;                    // of the single-step launch Ls
+    Tile *multi_d = nullptr;                    // CTA table of kind 9
+    long long multi_cap = 0;
+    int nmulti = 0;
     int grid = 0;
     int parity = 0;
     std::vector<char> dom_ready;
@@ -222,13 +225,19 @@ void drop_graph(vans_t h) {
     h->seg_graphs.clear();
 }
 
-// one batched step with the handle's launch (strip kernels for kinds 2, 4, 5)
+// one batched step with the handle's single-step launch (strip kernels for kinds
+// 2, 4, 5)
 cudaError_t batched_step(vans_t h, cudaStream_t s, int par) {
-    if (h->L.kind != 0)
-        return vans::launch_ring_batched(h->doms_d, h->tiles_d, (int)h->tiles.size(), par, h->L,
+    if (h->Ls.kind != 0)
+        return vans::launch_ring_batched(h->doms_d, h->tiles_d, (int)h->tiles.size(), par, h->Ls,
                                          h->flag + 1, s);
-    return vans::launch_step_batched(h->doms_d, h->tiles_d, (int)h->tiles.size(), par, h->L,
+    return vans::launch_step_batched(h->doms_d, h->tiles_d, (int)h->tiles.size(), par, h->Ls,
                                      h->grid, s);
+}
+
+// `steps` steps of the batch in one launch (kind 9)
+cudaError_t batched_multi(vans_t h, cudaStream_t s, int par, int steps) {
+    return vans::launch_multi_batched(h->doms_d, h->multi_d, h->nmulti, par, h->L.rows, steps, s);
 }
 
 // the single-step launch of a handle that nobody has tuned
@@ -237,7 +246,7 @@ Launch single_default(int q) { return q == 9 ? Launch{4, 4, 1, 0} : Launch{2, 4,
 // one launch of `steps` steps (more than one: kind 9)
 cudaError_t one_launch(vans_t h, cudaStream_t s, int par, int steps) {
     ++h->launches;
-    if (h->batched) return batched_step(h, s, par);
+    if (h->batched) return steps > 1 ? batched_multi(h, s, par, steps) : batched_step(h, s, par);
     if (steps > 1)
         return vans::launch_multi(h->dom, h->st[par], h->st[par ^ 1], steps, h->L.ctas, s);
     return vans::launch_step(h->q, h->dom, h->st[par], h->st[par ^ 1], h->Ls, s);
@@ -331,7 +340,7 @@ int run_single(vans_t h, int nsteps) {
 // 3 + 3 + 3, not 4 + 4 + 1: a launch of fewer steps saves less than it loses).
 // A single step is a single-step launch.
 int run_steps(vans_t h, int nsteps) {
-    if (h->batched || h->L.kind != 9 || h->slab || nsteps < 2) return run_single(h, nsteps);
+    if (h->L.kind != 9 || h->slab || nsteps < 2) return run_single(h, nsteps);
     const int most = h->L.rows, launches = (nsteps + most - 1) / most;
     const int few = nsteps / launches, longer = nsteps - few * launches;
     int rc = VANS_OK;
@@ -426,7 +435,45 @@ void build_tiles(vans_t h, const Launch &L, std::vector<Tile> &out) {
     }
 }
 
+// Kind 9: every domain cut into strips of about `rows` rows, four units (strip,
+// column block) per CTA, the longest strips first so that the last wave is short.
+// Long strips repeat fewer rows (6 per strip for 4 steps per launch), short ones
+// balance better: 256 channels of 64..1024 x 32..512 cells take 243 us per step
+// with strips of 96 rows, 249 with 48 and 263 with 192 (kind 4: 460).
+int multi_rows(const Launch &L) { return L.ctas == 1 ? 48 : L.ctas == 2 ? 192 : 96; }
+
+int set_batch_multi(vans_t h, const Launch &L) {
+    struct Cta {
+        Tile t;
+        int rows;
+    };
+    std::vector<Cta> ctas;
+    for (int d = 0; d < h->n; ++d) {
+        const VDom &D = h->doms[d];
+        if (!vans::multi_fits(9, D)) return VANS_ERR_UNSUPPORTED;
+        const int out = vans::multi_out_cols(L.rows), ncol = (D.nx + out - 1) / out;
+        const int nstrip = std::max(1, (D.ny + multi_rows(L) / 2) / multi_rows(L));
+        const long long units = (long long)ncol * nstrip;
+        if (units > 0x7fffffffLL - vans::kMultiWarps) return VANS_ERR_UNSUPPORTED;
+        for (long long u = 0; u < units; u += vans::kMultiWarps)
+            ctas.push_back(Cta{Tile{d, (int)u, ncol, nstrip}, (D.ny + nstrip - 1) / nstrip});
+    }
+    if ((long long)ctas.size() > h->multi_cap) return VANS_ERR_UNSUPPORTED;
+    std::stable_sort(ctas.begin(), ctas.end(),
+                     [](const Cta &a, const Cta &b) { return a.rows > b.rows; });
+    std::vector<Tile> t;
+    for (const Cta &c : ctas) t.push_back(c.t);
+    if (cudaMemcpyAsync(h->multi_d, t.data(), t.size() * sizeof(Tile), cudaMemcpyHostToDevice,
+                        h->stream) != cudaSuccess)
+        return VANS_ERR_CUDA;
+    h->nmulti = (int)t.size();
+    h->L = L;
+    drop_graph(h);
+    return VANS_OK;
+}
+
 int set_batch_launch(vans_t h, const Launch &L) {
+    if (L.kind == 9) return set_batch_multi(h, L);
     std::vector<Tile> t;
     build_tiles(h, L, t);
     if ((long long)t.size() > h->tile_cap) return VANS_ERR_ARG;
@@ -438,7 +485,7 @@ int set_batch_launch(vans_t h, const Launch &L) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     if (sms <= 0) sms = 1;
     h->grid = sms * vans::batched_blocks_per_sm(L);
-    h->L = L;
+    h->L = h->Ls = L;
     drop_graph(h);
     return VANS_OK;
 }
@@ -502,7 +549,9 @@ std::vector<Launch> candidates(int q, bool batched) {
                             {4, 4, 2, 5}, {4, 4, 3, 5}, {4, 4, 4, 5}, {2, 4, 2, 6}, {2, 8, 2, 6},
                             {4, 2, 4, 7}, {4, 2, 3, 7}, {4, 4, 2, 7}, {4, 4, 4, 7},
                             {4, 4, 2, 5, 2}, {4, 4, 2, 7, 2}, {4, 4, 3, 7, 2},
-                            {2, 4, 2, 2}, {2, 4, 4, 2}, {2, 4, 3, 4}};
+                            {2, 4, 2, 2}, {2, 4, 4, 2}, {2, 4, 3, 4},
+                            {2, 4, 4, 9, 0}, {2, 4, 4, 9, 1}, {2, 4, 4, 9, 2}, {2, 4, 3, 9, 0},
+                            {2, 4, 2, 9, 0}};
         c.insert(c.end(), std::begin(t), std::end(t));
         return c;
     }
@@ -753,8 +802,12 @@ int vans_set_launch(vans_t h, const vans_launch *cfg) {
     const Launch L{cfg->cpt, cfg->warps, cfg->rows, cfg->kind, cfg->ctas};
     if (!h->batched && h->dom.nee && !vans::launch_has_plates(h->q, L)) return VANS_ERR_UNSUPPORTED;
     if (L.kind == 8 && !vans::cluster_fits(h->q, h->dom, L.rows, L.warps)) return VANS_ERR_UNSUPPORTED;
-    if (L.kind == 9 && !h->slab && !vans::multi_fits(h->q, h->dom)) return VANS_ERR_UNSUPPORTED;
     if (h->batched) return set_batch_launch(h, L);
+    if (L.kind == 9) {
+        VDom whole = h->dom;         // a slab steps by single launches until the next vans_set_eps
+        whole.xwrap = 1;
+        if (!vans::multi_fits(h->q, whole)) return VANS_ERR_UNSUPPORTED;
+    }
     h->L = L;
     h->Ls = L.kind == 9 ? single_default(h->q) : L;
     drop_graph(h);
@@ -1049,10 +1102,19 @@ static long long batch_tile_cap(const vans_params *p, int n) {
     return t;
 }
 
+static long long batch_multi_cap(const vans_params *p, int n) {
+    long long t = 0;   // CTAs of kind 9 with strips of 48 rows, the shortest
+    const int out = vans::multi_out_cols(vans::kMultiMax), w = vans::kMultiWarps;
+    for (int d = 0; d < n; ++d)
+        t += ((long long)((p[d].nx + out - 1) / out) * ((p[d].ny + 47) / 48) + w - 1) / w;
+    return t;
+}
+
 size_t vans_batch_workspace_bytes(const vans_params *p, int n) {
     if (!p || n < 1) return 0;
     long long bytes = round_up((long long)n * sizeof(VDom), 256) +
-                      round_up(batch_tile_cap(p, n) * (long long)sizeof(Tile), 256);
+                      round_up(batch_tile_cap(p, n) * (long long)sizeof(Tile), 256) +
+                      round_up(batch_multi_cap(p, n) * (long long)sizeof(Tile), 256);
     for (int d = 0; d < n; ++d) {
         if (validate(&p[d], true) != VANS_OK) return 0;
         bytes += (2 * state_floats_of(9, p[d].nx, p[d].ny, 1) + eps_floats_of(9, p[d].nx, p[d].ny, 1)) *
@@ -1086,6 +1148,9 @@ int vans_batch_create(const vans_params *p, int n, void *workspace, size_t works
     h->tiles_d = (Tile *)w;
     h->tile_cap = batch_tile_cap(p, n);
     w += round_up(h->tile_cap * (long long)sizeof(Tile), 256);
+    h->multi_d = (Tile *)w;
+    h->multi_cap = batch_multi_cap(p, n);
+    w += round_up(h->multi_cap * (long long)sizeof(Tile), 256);
     h->doms.resize(n);
     long long dense = 0;
     for (int d = 0; d < n; ++d) {
@@ -1175,22 +1240,29 @@ int vans_batch_autotune(vans_t h, vans_launch *chosen) {
     if (!h || !h->batched) return VANS_ERR_ARG;
     for (int d = 0; d < h->n; ++d)
         if (!h->dom_ready[d]) return VANS_ERR_STATE;
-    const Launch keep = h->L;
-    Launch best = keep;
-    float best_ms = 1e30f;
+    Launch best = h->L, single = h->Ls;
+    float best_ms = 1e30f, single_ms = 1e30f;
     const int par = h->parity;
     for (const Launch &L : candidates(9, true)) {
         if (set_batch_launch(h, L) != VANS_OK) continue;
-        // reads the current parity and writes the other buffer of every domain
-        const float ms =
-            time_launches(h, [&](cudaStream_t st) { return batched_step(h, st, par); }, 5);
-        h->launches += 20;
+        // reads the current parity and writes the other buffer of every domain;
+        // scored per step
+        const int n = L.kind == 9 ? 2 : 5, steps = L.kind == 9 ? L.rows : 1;
+        const float ms = time_launches(h, [&](cudaStream_t st) {
+            return steps > 1 ? batched_multi(h, st, par, steps) : batched_step(h, st, par);
+        }, n) / (float)(n * steps);
+        h->launches += 4 * n;
         if (ms < best_ms) {
             best_ms = ms;
             best = L;
         }
+        if (steps == 1 && ms < single_ms) {
+            single_ms = ms;
+            single = L;
+        }
     }
-    int rc = set_batch_launch(h, best);
+    int rc = set_batch_launch(h, single);
+    if (!rc && best.kind == 9) rc = set_batch_launch(h, best);
     if (rc) return rc;
     if (cudaStreamSynchronize(h->stream) != cudaSuccess) return VANS_ERR_CUDA;
     if (chosen) {
@@ -1212,11 +1284,11 @@ int vans_batch_profile_step(vans_t h, unsigned long long *records_dev, long long
     if (capacity < 3 * n) return VANS_ERR_ARG;
     for (int d = 0; d < h->n; ++d)
         if (!h->dom_ready[d]) return VANS_ERR_STATE;
-    if (h->L.kind == 0) return VANS_ERR_UNSUPPORTED;
+    if (h->Ls.kind == 0) return VANS_ERR_UNSUPPORTED;
     if (cudaMemsetAsync(records_dev, 0, 3 * n * sizeof(unsigned long long), h->stream) != cudaSuccess)
         return VANS_ERR_CUDA;
     ++h->launches;
-    if (vans::launch_ring_batched(h->doms_d, h->tiles_d, (int)n, h->parity, h->L, h->flag + 1,
+    if (vans::launch_ring_batched(h->doms_d, h->tiles_d, (int)n, h->parity, h->Ls, h->flag + 1,
                                   h->stream, records_dev) != cudaSuccess)
         return VANS_ERR_CUDA;
     h->parity ^= 1;

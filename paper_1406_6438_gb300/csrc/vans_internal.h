@@ -133,6 +133,12 @@ cudaError_t launch_step_adjoint(int q, const VDom &d, const float *state, const 
                                 cudaStream_t stream);
 cudaError_t launch_grad_finalize(int q, const VDom &d, const float *lam0, const float *grad,
                                  float *dJ, cudaStream_t stream);
+// kind 9 over a batch: CTA table {dom, first of four units, column blocks, strips}
+// built for launches of table_steps steps, whose blocks store multi_out_cols columns
+constexpr int kMultiWarps = 4;
+int multi_out_cols(int steps);
+cudaError_t launch_multi_batched(const VDom *doms, const Tile *tiles, int ntiles, int parity,
+                                 int table_steps, int steps, cudaStream_t stream);
 // slabs along x: floats of one halo message, pack / unpack of the edge
 // columns' crossing populations, the porosity halo columns
 int halo_floats(int q, const VDom &d);

@@ -191,7 +191,6 @@ __device__ __forceinline__ void collide_pair(const VDom &d, const f2 h[9], const
     pair(8, 6, fma2(bc(-9.f), xy, b), sub2(qx, qy));
 }
 
-constexpr int kMultiWarps = 4;      // warps per block, each on its own
 constexpr int kPorBytes = 13 * 8 * 32;   // Por of one warp and row
 
 // columns on each side of a block that are computed but not stored: one per
@@ -236,9 +235,8 @@ __device__ __forceinline__ int wrap(int c, int n) {
 // wrap around like a periodic axis's and nothing of them is kept); what a row
 // next to a wall pulls from there is put in its place first: the entry that
 // bounced off, at the column from which the shift brings it home.
-template <int T, bool WALLS>
+template <int T, bool WALLS, int GL = ghost_cols(T)>
 struct Strip {
-    static constexpr int GL = ghost_cols(T);
     const VDom &d;
     const float *__restrict__ fin;
     float *__restrict__ fout;
@@ -293,12 +291,12 @@ struct Strip {
         raw[4] = load(fin + 4 * plane, op);
         raw[7] = load(fin + 7 * plane, op);
         raw[8] = load(fin + 8 * plane, op);
-        if (W && y == 0) {
+        if (W && d.wall_y && y == 0) {
             raw[2] = load(fin + 4 * plane, oz);
             raw[5] = load_beside(fin + 7 * plane, y, 1);
             raw[6] = load_beside(fin + 8 * plane, y, -1);
         }
-        if (W && y == d.ny - 1) {
+        if (W && d.wall_y && y == d.ny - 1) {
             raw[4] = load(fin + 2 * plane, oz);
             raw[7] = load_beside(fin + 5 * plane, y, -1);
             raw[8] = load_beside(fin + 6 * plane, y, 1);
@@ -332,8 +330,8 @@ struct Strip {
         h[7] = from_right(raw[7]);
         h[8] = from_left(raw[8]);
         Por P;
-        const bool above = W && r == d.ny - 1;
-        porosity_terms(d, em, ez, ep, W && r == 0, above, P);
+        const bool above = W && d.wall_y && r == d.ny - 1;
+        porosity_terms(d, em, ez, ep, W && d.wall_y && r == 0, above, P);
         por_put(por_row(slot), lane, P);
         em = ez;
         ez = ep;
@@ -416,7 +414,7 @@ struct Strip {
             // the next turn's row, before the last step: earlier, the twenty
             // registers it lands in would be live through every step
             if (l == T - 1 && more) prefetch<W>();
-            if (W && r - l + 1 == d.ny) {  // past the upper wall: row ny-1 bounced
+            if (W && d.wall_y && r - l + 1 == d.ny) {  // past the upper wall: row ny-1 bounced
                 const f2 *u = up_row(l, odd ^ 1);
                 o[4] = u[0 * 32];
                 o[7] = u[1 * 32];
@@ -425,7 +423,7 @@ struct Strip {
             f2 on[9];
             if (l < N) next<W>(l, o, on);
             keep(l, o);
-            if (W && r - l + 1 == 0) {     // below the lower wall: row 0 bounced
+            if (W && d.wall_y && r - l + 1 == 0) {     // below the lower wall: row 0 bounced
                 f2 *u = up_row(l, odd ^ 1);
                 u[0 * 32] = o[4];
                 u[1 * 32] = o[7];
@@ -455,7 +453,7 @@ struct Strip {
     __device__ __forceinline__ void run(int xs) {
         x = xs - GL + 2 * lane;                        // the lane's first column
         inside = xs - GL >= 0 && xs - GL + 64 <= d.nx;
-        xedge = xs == 0 || xs + out_cols(T) >= d.nx;
+        xedge = xs == 0 || xs + 64 - 2 * GL >= d.nx;
         ia = inside ? x : wrap(x, d.nx);
         second = inside ? 4u : (uint32_t)(wrap(x + 1, d.nx) - ia) * 4u;
         slot = 0;
@@ -506,23 +504,47 @@ __host__ __device__ constexpr int warp_smem() {
     return T * kPorBytes + (T - 1) * 2 * 3 * 8 * 32;
 }
 
-// Unit (strip, column block) of this warp.
+// The strip and column block of unit `unit` of a domain cut into ncol x nstrip.
+template <int T, bool WALLS, int GL>
+__device__ __forceinline__ void run_unit(const VDom &d, const float *fin, float *fout, int unit,
+                                         int ncol, int nstrip, unsigned char *smem) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int strip = unit / ncol, col = unit - strip * ncol;
+    unsigned char *ring = smem + warp * warp_smem<T>();
+    f2 *up = reinterpret_cast<f2 *>(ring + T * kPorBytes) + lane;
+    Strip<T, WALLS, GL> s{d, fin, fout, ring, up};
+    s.y0 = (int)((long long)strip * d.ny / nstrip);
+    s.y1 = (int)((long long)(strip + 1) * d.ny / nstrip);
+    s.lane = lane;
+    s.run(col * (64 - 2 * GL));
+}
+
 template <int T, bool WALLS>
 __global__ void __launch_bounds__(32 * kMultiWarps, 3)
     k_multi(const VDom d, const float *__restrict__ fin, float *__restrict__ fout, int ncol,
             int nstrip) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int unit = blockIdx.x * kMultiWarps + warp;
+    const int unit = blockIdx.x * kMultiWarps + (threadIdx.x >> 5);
     if (unit >= ncol * nstrip) return;
-    const int strip = unit / ncol, col = unit - strip * ncol;
-    unsigned char *ring = smem + warp * warp_smem<T>();
-    f2 *up = reinterpret_cast<f2 *>(ring + T * kPorBytes) + lane;
-    Strip<T, WALLS> s{d, fin, fout, ring, up};
-    s.y0 = (int)((long long)strip * d.ny / nstrip);
-    s.y1 = (int)((long long)(strip + 1) * d.ny / nstrip);
-    s.lane = lane;
-    s.run(col * out_cols(T));
+    run_unit<T, WALLS, ghost_cols(T)>(d, fin, fout, unit, ncol, nstrip, smem);
+}
+
+// Batched: block b takes four consecutive units of one domain, table entry {dom,
+// first unit, column blocks, strips}.  GL: ghost columns that the table was built
+// for (a remainder of fewer steps runs on the table of the full launches).
+template <int T, int GL>
+__global__ void __launch_bounds__(32 * kMultiWarps, 3)
+    k_multi_batched(const VDom *__restrict__ doms, const Tile *__restrict__ tiles, int parity) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ VDom d;
+    const Tile t = tiles[blockIdx.x];
+    for (int k = threadIdx.x; k < (int)(sizeof(VDom) / 4); k += blockDim.x)
+        reinterpret_cast<int *>(&d)[k] = reinterpret_cast<const int *>(doms + t.dom)[k];
+    __syncthreads();
+    const int unit = t.row + (threadIdx.x >> 5);
+    if (unit >= t.x0 * t.pad) return;
+    run_unit<T, true, GL>(d, parity ? d.f[1] : d.f[0], parity ? d.f[0] : d.f[1], unit, t.x0, t.pad,
+                          smem);
 }
 
 template <int T, bool WALLS>
@@ -572,6 +594,32 @@ cudaError_t launch_steps(const VDom &d, const float *fin, float *fout, int ctas,
 }
 
 }  // namespace
+
+template <int T, int GL>
+static cudaError_t launch_batched_t(const VDom *doms, const Tile *tiles, int ntiles, int parity,
+                                    cudaStream_t stream) {
+    auto kern = k_multi_batched<T, GL>;
+    const size_t smem = (size_t)kMultiWarps * warp_smem<T>();
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<ntiles, 32 * kMultiWarps, smem, stream>>>(doms, tiles, parity);
+    return cudaGetLastError();
+}
+
+int multi_out_cols(int steps) { return out_cols(steps); }
+
+cudaError_t launch_multi_batched(const VDom *doms, const Tile *tiles, int ntiles, int parity,
+                                 int table_steps, int steps, cudaStream_t stream) {
+    if (ntiles < 1) return cudaErrorInvalidValue;
+    if (table_steps == 2 && steps == 2) return launch_batched_t<2, 2>(doms, tiles, ntiles, parity, stream);
+    if (table_steps < 3) return cudaErrorInvalidValue;
+    switch (steps) {
+        case 2: return launch_batched_t<2, 4>(doms, tiles, ntiles, parity, stream);
+        case 3: return launch_batched_t<3, 4>(doms, tiles, ntiles, parity, stream);
+        case 4: return launch_batched_t<4, 4>(doms, tiles, ntiles, parity, stream);
+    }
+    return cudaErrorInvalidValue;
+}
 
 bool multi_fits(int q, const VDom &d) {
     // byte offsets within a plane are 32-bit

@@ -86,3 +86,29 @@ def test_single_steps_and_refusals():
     with pytest.raises(VansError) as e:
         solver(q, epsc, Launch(2, 4, 2, 9))
     assert e.value.status == -5
+
+
+@pytest.mark.parametrize("L", [Launch(2, 4, 2, 9), Launch(2, 4, 3, 9, 1), Launch(2, 4, 4, 9, 1),
+                               Launch(2, 4, 4, 9, 2)])
+@pytest.mark.parametrize("nsteps", [5, 14])
+def test_batch_matches_oracle(L, nsteps):
+    """Uneven domains (walls, moving wall, periodic; one of a single row and column,
+    one of several strips) in one batch, each against the oracle."""
+    torch = torch_cuda()
+    import paper_1406_6438_gb300 as V
+    cases = [_case(ny, nx, w, m, k, seed=ny) for ny, nx, w, m, k in
+             [(40, 130, True, False, 0), (1, 1, True, False, 0), (150, 61, True, True, 1),
+              (33, 300, False, False, 2), (97, 56, True, False, 2), (5, 20, False, False, 0)]]
+    b = V.Batch([p for p, _, _ in cases])
+    for d, (_, eps, _) in enumerate(cases):
+        b.set_eps(d, torch.from_numpy(eps).cuda().view(-1))
+    b.launch = L
+    b.step(nsteps)
+    for d, (p, eps, _) in enumerate(cases):
+        rho_o, u_o, f_o = oracle_run(p, eps, nsteps)
+        rho, u = b.moments(d)
+        f = b.populations(d)
+        torch.cuda.synchronize()
+        assert np.abs(f.cpu().numpy() - f_o).max() <= 2e-7, (d, L)
+        assert rel_u(u.cpu().numpy(), u_o) <= 1e-5, (d, L)
+    assert b.launch == L
