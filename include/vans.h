@@ -198,10 +198,10 @@ int vans_update_eps(vans_t h, const float *eps_dev);
  * vans_set_eps, VANS_ERR_ARG for nsteps < 0, VANS_ERR_CUDA. */
 int vans_step(vans_t h, int nsteps);
 
-/* vans_step by launches of one step each (or the one launch of kind 8), whatever
- * launch configuration is set: the forward run of a checkpointed reverse pass.
+/* vans_step by launches of one step each (or the one launch of kind 8, in a form
+ * that rounds like them): the forward run of a checkpointed reverse pass.
  * vans_adjoint_segment recomputes its states with the same launches, bit for bit;
- * those of a run of several steps per launch (kind 9) differ by FP32 roundings.
+ * those of vans_step with kinds 8 and 9 differ by FP32 roundings.
  * Errors as vans_step. */
 int vans_step_single(vans_t h, int nsteps);
 

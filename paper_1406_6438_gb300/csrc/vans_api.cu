@@ -275,20 +275,6 @@ int capture_launches(vans_t h, int n, int steps, cudaGraphExec_t *out) {
     return VANS_OK;
 }
 
-// all graph sizes at once, so the first run that needs any of them pays the
-// capture for every later run length
-int ensure_graphs(vans_t h, cudaGraphExec_t *gs, int steps) {
-    if (gs[0]) return VANS_OK;
-    for (int k = 0; k < kGraphSizes; ++k) {
-        const int rc = capture_launches(h, kGraphSteps >> k, steps, &gs[k]);
-        if (rc) {
-            drop_graph(h);
-            return rc;
-        }
-    }
-    return VANS_OK;
-}
-
 // `count` launches of `steps` steps each, replayed from the graphs gs (nullptr:
 // launched one by one); the parity lives in h->cur (single) or h->parity (batched)
 int run_launches(vans_t h, int count, int steps, cudaGraphExec_t *gs) {
@@ -301,11 +287,18 @@ int run_launches(vans_t h, int count, int steps, cudaGraphExec_t *gs) {
             --left;
         }
         if (left >= 2) {
-            int rc = ensure_graphs(h, gs, steps);
-            if (rc) return rc;
+            // a size is captured when a run first needs it: all six at once are 126
+            // launches, of which a short run replays a few
             for (int k = 0; k < kGraphSizes; ++k) {
                 const int n = kGraphSteps >> k;
                 while (left >= n) {
+                    if (!gs[k]) {
+                        const int rc = capture_launches(h, n, steps, &gs[k]);
+                        if (rc) {
+                            drop_graph(h);
+                            return rc;
+                        }
+                    }
                     if (cudaGraphLaunch(gs[k], h->stream) != cudaSuccess) return VANS_ERR_CUDA;
                     h->launches += n;
                     left -= n;
@@ -321,17 +314,21 @@ int run_launches(vans_t h, int count, int steps, cudaGraphExec_t *gs) {
     return VANS_OK;
 }
 
-// nsteps steps by single-step launches (kind 8: all of them in one launch)
+// nsteps steps in one launch of the cluster-resident kind 8; the result lands where
+// the step-by-step run would leave it
+int run_cluster(vans_t h, int nsteps, const Launch &L, bool pairs) {
+    ++h->launches;
+    if (vans::launch_step_cluster(h->q, h->dom, h->st[h->cur], h->st[h->cur ^ (nsteps & 1)], nsteps,
+                                  L, pairs, h->stream) != cudaSuccess)
+        return VANS_ERR_CUDA;
+    h->cur ^= nsteps & 1;
+    return VANS_OK;
+}
+
+// nsteps steps by single-step launches, or by the one launch of kind 8 in the form
+// that rounds like them: the forward run of a reverse pass
 int run_single(vans_t h, int nsteps) {
-    if (!h->batched && h->Ls.kind == 8 && nsteps > 0) {
-        // the result lands where the step-by-step run would leave it
-        ++h->launches;
-        if (vans::launch_step_cluster(h->q, h->dom, h->st[h->cur], h->st[h->cur ^ (nsteps & 1)],
-                                      nsteps, h->Ls, h->stream) != cudaSuccess)
-            return VANS_ERR_CUDA;
-        h->cur ^= nsteps & 1;
-        return VANS_OK;
-    }
+    if (!h->batched && h->Ls.kind == 8 && nsteps > 0) return run_cluster(h, nsteps, h->Ls, false);
     return run_launches(h, nsteps, 1, h->gexec);
 }
 
@@ -340,6 +337,7 @@ int run_single(vans_t h, int nsteps) {
 // 3 + 3 + 3, not 4 + 4 + 1: a launch of fewer steps saves less than it loses).
 // A single step is a single-step launch.
 int run_steps(vans_t h, int nsteps) {
+    if (!h->batched && h->L.kind == 8 && nsteps > 0) return run_cluster(h, nsteps, h->L, true);
     if (h->L.kind != 9 || h->slab || nsteps < 2) return run_single(h, nsteps);
     const int most = h->L.rows, launches = (nsteps + most - 1) / most;
     const int few = nsteps / launches, longer = nsteps - few * launches;
@@ -845,21 +843,21 @@ int vans_autotune(vans_t h, vans_launch *chosen) {
             continue;
         }
         if (L.kind == 8) {
-            // kind 8 runs the steps of a call in one launch: of reps steps, and of
-            // five times as many for the comparison with kind 9 (odd counts: the
-            // result lands in the spare buffer, as one step of the other kinds does)
-            auto steps = [&](int n) {
+            // kind 8 runs the steps of a call in one launch: of five times reps steps
+            // for a run, of reps in the form of the single-step kinds (odd counts:
+            // the result lands in the spare buffer, as one step of theirs does)
+            auto steps = [&](int n, bool pairs) {
                 h->launches += 4;
                 return time_launches(h, [&](cudaStream_t st) {
-                    return vans::launch_step_cluster(h->q, h->dom, in, outb, n, L, st);
+                    return vans::launch_step_cluster(h->q, h->dom, in, outb, n, L, pairs, st);
                 }, 1);
             };
-            const float many = steps(5 * reps) / 5.f;
+            const float many = steps(5 * reps, true) / 5.f;
             if (many < best_ms) {
                 best_ms = many;
                 best = L;
             }
-            ms = steps(reps);
+            ms = steps(reps, false);
         } else {
             ms = time_launches(h, [&](cudaStream_t st) {
                 return vans::launch_step(h->q, h->dom, in, outb, L, st);
@@ -877,7 +875,7 @@ int vans_autotune(vans_t h, vans_launch *chosen) {
     }
     if (cudaGetLastError() != cudaSuccess) return VANS_ERR_CUDA;
     h->L = best;
-    h->Ls = best.kind == 9 ? single : best;
+    h->Ls = best.kind >= 8 ? single : best;
     drop_graph(h);
     if (chosen) {
         chosen->cpt = best.cpt;

@@ -87,9 +87,11 @@ cudaError_t launch_monitor_finalize(const float *part, float *stats, cudaStream_
 cudaError_t launch_step_tma(int q, const VDom &d, const float *fin, float *fout, Launch L,
                             cudaStream_t stream);
 // kind 8: nsteps steps in one launch of one thread-block cluster that holds the
-// whole state in its shared memory; reads fin, writes fout (which may be fin)
+// whole state in its shared memory; reads fin, writes fout (which may be fin).
+// pairs: D2Q9 domains that fit take the form with two cells per thread (packed
+// arithmetic: other roundings than the single-step kinds)
 cudaError_t launch_step_cluster(int q, const VDom &d, const float *fin, float *fout, int nsteps,
-                                Launch L, cudaStream_t stream);
+                                Launch L, bool pairs, cudaStream_t stream);
 // kind 9 (D2Q9, x periodic within the domain, no plates on nodes): `steps`
 // (2..kMultiMax) steps in one launch, in strips for `ctas` CTAs per SM (0: chosen)
 constexpr int kMultiMax = 4;

@@ -79,13 +79,29 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
     return ok != 0;
 }
 
+// the same with acquire semantics over the cluster: for barriers that other CTAs'
+// st.async writes complete
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t *bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_addr(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 // Wait for phase `parity` of `bar`, giving up after ~1 s (2^31 SM cycles) or
 // 2^24 polls, whichever comes first.  Returns false on timeout.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity) {
-    if (mbar_try_wait(bar, parity)) return true;
+    auto done = [&] { return CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity); };
+    if (done()) return true;
     const long long t0 = clock64();
     for (int it = 0; it < (1 << 24); ++it) {
-        if (mbar_try_wait(bar, parity)) return true;
+        if (done()) return true;
         if (clock64() - t0 > (1LL << 31)) break;
     }
     return false;

@@ -99,3 +99,33 @@ def test_porous_couette_of_the_paper_in_one_cluster_launch(Re, Da):
     assert rel_u(u, u_o) <= 1e-5, rel_u(u, u_o)
     assert np.abs(f - f_o).max() <= 2e-7
     assert np.abs(f - f_ref).max() <= 6e-8
+
+
+PAIR_CASES = [
+    # (ny, nx): one cell, one column, one row; a band per row; a last band of one row;
+    # odd rows (a last pair of one cell); rows that straddle warps
+    ((1, 1), 0, {}), ((1, 2), 2, {}), ((3, 1), 0, {}), ((2, 7), 2, dict(u_wall=(0.02, 0.0, 0.0))),
+    ((16, 6), 0, {}), ((17, 33), 0, {}), ((33, 31), 2, dict(u_wall=(0.01, 0.004, 0.0))),
+    ((12, 81), 0, {}), ((64, 16), 2, {}),
+    # plates on nodes alone in their bands, and in one band with their neighbours
+    ((3, 9), 2, dict(wall_kind=1, u_wall=(0.01, 0.0, 0.0))),
+    ((16, 10), 2, dict(wall_kind=1, u_wall=(0.01, 0.0, 0.0))),
+    ((17, 41), 2, dict(wall_kind=1, u_wall=(0.01, 0.0, 0.0))),
+    # more pairs than threads (33 rows of 8 pairs on 8 warps): the one-cell form
+    ((66, 15), 0, {}),
+]
+
+
+@pytest.mark.parametrize("shape,wm,kw", PAIR_CASES)
+@pytest.mark.parametrize("nsteps", [1, 2, 11])
+def test_pair_form_matches_the_oracle(shape, wm, kw, nsteps):
+    """The D2Q9 pair form at the edges of its bands, rows and copies (odd and even
+    step counts end in either copy); tolerance as for every step kernel."""
+    p, eps, f0 = _case(9, (1,) + shape, wm, **kw)
+    rho_o, u_o, f_o = oracle_run(p, eps, nsteps, f0)
+    for L in (Launch(1, 8, 16, 8), Launch(1, 16, 5, 8), Launch(1, 8, 2, 8)):
+        if -(-shape[0] // L.rows) * shape[1] > 64 * L.warps:
+            continue                                  # does not fit this cluster
+        rho, u, f = gpu_run(p, eps, nsteps, f0, launch=L)
+        assert np.abs(f - f_o).max() <= 2e-7, (L, np.abs(f - f_o).max())
+        assert rel_u(u, u_o) <= 1e-5, L
