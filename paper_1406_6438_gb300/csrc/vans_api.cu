@@ -105,7 +105,7 @@ bool launch_ok(const vans_launch *c, int q, bool batched) {
         return (nt == 64 || nt == 128) && c->cpt == (q == 9 ? 4 : 2) && (q == 9 || !batched);
     if (c->kind == 6)
         return q == 9 ? (c->cpt == 2 && (nt == 128 || nt == 256))
-                      : (c->cpt == 1 && (nt == 128 || nt == 256) && !batched);
+                      : (c->cpt == 1 && c->warps >= 2 && c->warps <= 8 && !batched);
     if (q == 9)
         return (nt == 128 && (c->cpt == 2 || c->cpt == 4)) || (nt == 256 && c->cpt <= 2);
     return (nt == 128 && c->cpt <= 2) || (nt == 256 && c->cpt == 1);
@@ -571,6 +571,9 @@ std::vector<Launch> candidates(int q, bool batched) {
                             {2, 4, 2, 5, 2}, {2, 2, 2, 7}, {2, 2, 4, 7}, {2, 6, 2, 7},
                             {2, 3, 2, 7}, {2, 3, 3, 7}, {2, 5, 2, 7}};
         c.insert(c.end(), std::begin(t), std::end(t));
+        for (int stages = 2; stages <= 3; ++stages)
+            for (int warps = 2; warps <= 8; ++warps)
+                if (!(stages == 3 && warps % 4 == 0)) c.push_back(Launch{1, warps, stages, 6});
     }
     // cluster-resident multi-step shapes {1, warps, largest cluster, 8}; the
     // autotuner skips those whose cluster cannot hold the domain
@@ -827,6 +830,13 @@ int vans_autotune(vans_t h, vans_launch *chosen) {
         if (h->dom.nee && !vans::launch_has_plates(h->q, L)) continue;   // no plate instance
         if (L.kind == 8 && !vans::cluster_fits(h->q, h->dom, L.rows, L.warps)) continue;
         if (L.kind == 9 && !vans::multi_fits(h->q, h->dom)) continue;
+        // D3Q19, one cell per thread: of the tile widths only the one that takes a row
+        // in the fewest tiles with the fewest idle lanes (beside 128 and 256 cells with
+        // 3 stages).  150 x 110 x 90: 160 cells 45.0 us, 192 51, 224 62, 96 (two tiles) 61
+        const int tiles = (h->dom.nx + 255) / 256, cells = (h->dom.nx + tiles - 1) / tiles;
+        if (h->q == 19 && L.kind == 6 && (L.rows == 2 || L.warps % 4 != 0) &&
+            (cells + 31) / 32 != L.warps)
+            continue;
         // all scored as the time of `reps` steps
         float ms = 1e30f;
         if (L.kind == 9) {

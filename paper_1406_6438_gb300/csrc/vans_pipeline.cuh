@@ -51,11 +51,11 @@ __host__ __device__ constexpr uint32_t seg_bytes(int nval) {
 // thread): the Q population rows the pull reads and the porosity rows.  The
 // barrier's transaction count also covers `extra` further copies of the same
 // size, which the caller issues; the size of each copy is returned.
-// WRAP (rows that are one tile, nx a multiple of 8, column 0 on a 128-byte
-// line): only the cells are copied, whole lines and no halo columns, which the
-// compute then takes from the other end of the staged row (the periodic x wrap:
-// every write of a halo entry also writes its mirror there); a segment with
-// halos touches one more 128-byte line per row, 12 % more reads on 256-cell
+// WRAP (rows that are one tile, column 0 on a 128-byte line): the cells are copied
+// in whole sectors from column 0 on, and the compute takes column -1, and column nx
+// where nx is a multiple of 8, from the other end of the staged row (the periodic x
+// wrap: every write of a halo entry also writes its mirror there); a segment with
+// halos touches one or two more 128-byte lines per row, 12 % more reads on 256-cell
 // rows.
 template <int Q, int TW, bool WRAP = false>
 __device__ __forceinline__ uint32_t issue_tile(const VDom &d, const float *__restrict__ fin, int row,
@@ -67,7 +67,7 @@ __device__ __forceinline__ uint32_t issue_tile(const VDom &d, const float *__res
     Nb3 Y, Z;
     row_nbs<Q>(d, row, y, z, Y, Z);
     const int nval = min(TW, d.nx - xs);
-    const uint32_t bytes = WRAP ? (uint32_t)(nval * 4) : seg_bytes(nval);
+    const uint32_t bytes = WRAP ? (uint32_t)(((nval + 7) & ~7) * 4) : seg_bytes(nval);
     const int c0 = WRAP ? xs : xs - kLead;        // first column copied
     const int s0 = WRAP ? kLead : 0;              // its place in the stage row
     mbar_arrive_expect_tx(bar, bytes * (NS + extra));

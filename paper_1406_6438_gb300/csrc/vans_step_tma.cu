@@ -22,7 +22,14 @@
 //      stores).
 //   6, 7  k_step_tma_ilv: persistent CTAs take tiles b, b+G, ... of the
 //      row-major order (the whole grid sweeps one band of rows), warp-
-//      specialised as 4/5; 6 strided cells, 7 adjacent cells.
+//      specialised as 4/5; 6 strided cells, 7 adjacent cells.  D3Q19 domains
+//      whose rows are not 256 cells are bound by too few warps for the
+//      arithmetic (12 per SM of kind 7 with 2 cells per thread, 127 registers)
+//      and by idle lanes: kind 6 takes one cell per thread (76 registers, 20
+//      warps) in tiles of 64 to 256 cells, rows of one tile without the staged
+//      halo columns: 150 x 110 x 90 58 -> 45 us (floor 34), 250^3 459 -> 392
+//      (360), 90^3 43 -> 27, 96 x 64 x 48 14.9 -> 11.6; 256^3 stays with kind 7
+//      (397 against 414).
 //
 // (Kinds 1 -- a pipeline over contiguous runs of tiles with the porosity rows
 // staged per tile -- and 3 -- kind 2 with adjacent cells -- were never the
@@ -264,10 +271,12 @@ __device__ __forceinline__ void ring_tile(const VDom &d, const float *__restrict
 #pragma unroll
         for (int cc = 0; cc < CPT; ++cc) {
             const int xl = tid + cc * NT;
+            const int xm = WRAP && xl == 0 ? d.nx - 1 : xl - 1;
+            const int xp = WRAP && xl == d.nx - 1 ? 0 : xl + 1;
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
                 const bool bb = ywall(1 - L::ey(i)) || zwall(1 - L::ez(i));
-                h[cc][i] = sb[i * SEG + kLead + xl + (bb ? 0 : -L::ex(i))];
+                h[cc][i] = sb[i * SEG + kLead + (bb || L::ex(i) == 0 ? xl : L::ex(i) > 0 ? xm : xp)];
             }
             const float e0 = ey_slot[1][(Q == 9 ? 0 : 1) * SEG + kLead + xl];
             et[cc][0] = e0;
@@ -276,7 +285,8 @@ __device__ __forceinline__ void ring_tile(const VDom &d, const float *__restrict
                 const int ey = L::ey(i), ez = L::ez(i);
                 const bool wall = ywall(1 + ey) || zwall(1 + ez);
                 et[cc][i] =
-                    wall ? e0 : ey_slot[1 + ey][(Q == 9 ? 0 : 1 + ez) * SEG + kLead + xl + L::ex(i)];
+                    wall ? e0 : ey_slot[1 + ey][(Q == 9 ? 0 : 1 + ez) * SEG + kLead +
+                                                (L::ex(i) == 0 ? xl : L::ex(i) > 0 ? xp : xm)];
             }
         }
         release();
@@ -322,6 +332,8 @@ __device__ __forceinline__ void ring_tile(const VDom &d, const float *__restrict
                     for (int i = 0; i < Q; ++i)
                         if (L::ex(i) > 0) store_halo_lo<Q>(fout + i * d.plane + ro, o[i]);
                 }
+            } else if (in_row_tail<Q>(d.nx, x)) {
+                store_row_tail<Q>(fout, d.plane, ro, d.nx, x);
             }
         }
     }
@@ -715,10 +727,11 @@ static cudaError_t launch_ilv_t(const VDom &d, const float *fin, float *fout, in
     const size_t smem = kBarBytes + (size_t)stages * NS * (TW + 2 * kLead) * sizeof(float);
     if (stages < 2 || stages > kBarBytes / 16 || smem > 227 * 1024) return cudaErrorInvalidValue;
     const size_t smem_req = cap_smem(smem, ctas);
-    // D3Q19 rows that are one tile, nx a multiple of 8, x periodic within the
-    // domain (not a slab): cells-only staging
-    constexpr bool kWrapOk = Q == 19 && VEC && !PL;
-    const bool wrap = kWrapOk && d.nx <= TW && (d.nx & 7) == 0 && d.off == 32 && d.xwrap;
+    // D3Q19 rows that are one tile, x periodic within the domain (not a slab):
+    // cells-only staging; with adjacent cells per thread nx a multiple of 8 (with the
+    // code for other rows 256^3 took 422 us instead of 411, and kind 6 is faster there)
+    constexpr bool kWrapOk = Q == 19 && !PL;
+    const bool wrap = kWrapOk && d.nx <= TW && (!VEC || (d.nx & 7) == 0) && d.off == 32 && d.xwrap;
     auto kern = wrap ? k_step_tma_ilv<Q, NT, CPT, VEC, PL, kWrapOk>
                      : k_step_tma_ilv<Q, NT, CPT, VEC, PL, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_req);
@@ -936,6 +949,12 @@ cudaError_t launch_step_tma(int q, const VDom &d, const float *fin, float *fout,
         if (q == 9 && nt == 256 && L.cpt == 2) return launch_ilv_t<9, 256, 2, false>(d, fin, fout, L.rows, L.ctas, stream);
         if (q == 19 && nt == 128 && L.cpt == 1) return launch_ilv_t<19, 128, 1, false>(d, fin, fout, L.rows, L.ctas, stream);
         if (q == 19 && nt == 256 && L.cpt == 1) return launch_ilv_t<19, 256, 1, false>(d, fin, fout, L.rows, L.ctas, stream);
+        // the other widths, for D3Q19 rows that are one tile (vans_autotune)
+        if (q == 19 && nt == 64 && L.cpt == 1) return launch_ilv_t<19, 64, 1, false>(d, fin, fout, L.rows, L.ctas, stream);
+        if (q == 19 && nt == 96 && L.cpt == 1) return launch_ilv_t<19, 96, 1, false>(d, fin, fout, L.rows, L.ctas, stream);
+        if (q == 19 && nt == 160 && L.cpt == 1) return launch_ilv_t<19, 160, 1, false>(d, fin, fout, L.rows, L.ctas, stream);
+        if (q == 19 && nt == 192 && L.cpt == 1) return launch_ilv_t<19, 192, 1, false>(d, fin, fout, L.rows, L.ctas, stream);
+        if (q == 19 && nt == 224 && L.cpt == 1) return launch_ilv_t<19, 224, 1, false>(d, fin, fout, L.rows, L.ctas, stream);
         return cudaErrorInvalidValue;
     }
     if (L.kind == 7) {                  // interleaved tiles, consecutive cells per thread
