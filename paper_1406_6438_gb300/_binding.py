@@ -402,8 +402,9 @@ class Solver:
         return torch.zeros(self.state_floats, dtype=torch.float32, device=self.device)
 
     def get_state(self, out=None):
+        torch = _torch()
         if out is None:
-            out = self.new_state()
+            out = torch.empty(self.state_floats, dtype=torch.float32, device=self.device)
         _check(self.lib.vans_get_state(self._h, _f32(out, self.state_floats, "state")),
                "vans_get_state")
         return out

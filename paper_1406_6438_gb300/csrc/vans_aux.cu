@@ -1,6 +1,8 @@
 // vans_aux.cu -- everything around the step: porosity set-up, moments, state
 // import/export, divergence check, outlet flux, and the register-load form of
 // the reverse-mode adjoint step (the pipelined one is in vans_adjoint_tma.cu).
+#include <cooperative_groups.h>
+
 #include "vans_adjoint.cuh"
 #include "vans_device.cuh"
 
@@ -278,12 +280,18 @@ __global__ void k_check(const VDom d, const float *__restrict__ st, int *flag) {
 
 // ------------------------------------------------------ reverse mode -----
 
-// J = sum over the plane x = x_out of eps rho u_x; one block, fixed-order sum.
+// J = sum over the plane x = x_out of eps rho u_x, summed in a fixed order by one
+// cluster of blocks: the plane's entries are a sector each, and one block of 256
+// threads waited for 12 rounds of them on 64 x 48 rows (67 us, now 15).
+constexpr int kFluxBlocks = 8;
 template <int Q>
-__global__ void __launch_bounds__(256) k_flux(const VDom d, const float *__restrict__ st, int x_out, float *J) {
+__global__ void __cluster_dims__(kFluxBlocks, 1, 1) __launch_bounds__(256)
+    k_flux(const VDom d, const float *__restrict__ st, int x_out, float *J) {
+    namespace cg = cooperative_groups;
     __shared__ float red[256];
+    cg::cluster_group cluster = cg::this_cluster();
     float acc = 0.f;
-    for (int r = threadIdx.x; r < d.rows; r += blockDim.x) {
+    for (int r = blockIdx.x * 256 + threadIdx.x; r < d.rows; r += kFluxBlocks * 256) {
         const int y = r % d.ny, z = r / d.ny;
         Nb3 Y, Z;
         nb_yz<Q>(d, y, z, Y, Z);
@@ -300,7 +308,13 @@ __global__ void __launch_bounds__(256) k_flux(const VDom d, const float *__restr
         if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
         __syncthreads();
     }
-    if (threadIdx.x == 0) J[0] = red[0];
+    cluster.sync();
+    if (cluster.block_rank() == 0 && threadIdx.x == 0) {
+        float v = 0.f;
+        for (int b = 0; b < kFluxBlocks; ++b) v += *cluster.map_shared_rank(red, b);
+        J[0] = v;
+    }
+    cluster.sync();                     // no block leaves while its sum is read
 }
 
 // Seed of the reverse pass: lambda at the entries the outlet cells pull, and
@@ -466,51 +480,80 @@ __global__ void __launch_bounds__(256) k_step_adjoint(const VDom d, const float 
         adj_row<Q, CPT, false, T>(d, st, lin, lout, grad, y, z, x0, lane);
 }
 
+// A sum held as two floats, head and tail (Knuth's two-sum; 48 bits).
+struct TwoFloat {
+    float h = 0.f, l = 0.f;
+    __device__ __forceinline__ void add(float a) {
+        const float s = h + a, b = s - h;
+        l += (h - (s - b)) + (a - b);
+        h = s;
+    }
+    // w times the sum t, the rounding of w * t.h included
+    __device__ __forceinline__ void add_scaled(float w, const TwoFloat &t) {
+        const float p = w * t.h;
+        add(p);
+        l += fmaf(w, t.h, -p) + w * t.l;
+    }
+};
+
 // dJ/deps = G_eps + sum_i w_i lambda_i(0) (from f(0) = w eps) + the transposed
-// grad-eps stencil applied to G_grad.  Runs once per reverse pass; it combines
-// each compensated accumulator (sum + compensation) and evaluates the stencil,
-// whose terms cancel to a much smaller result, in FP64.
+// grad-eps stencil applied to G_grad.  Runs once per reverse pass; the stencil's
+// terms cancel to a much smaller result, so it combines the compensated accumulators
+// (sum + compensation) and evaluates the stencil as two-float sums, one per weight
+// (axis and diagonal directions), scaled at the end.  In FP64 the kernel was bound by
+// that pipe, of 1/64 of the FP32 rate: 96 x 64 x 48 175 us, 512^2 59 us (now 38, 14).
 template <int Q>
-__global__ void k_grad_finalize(const VDom d, const float *__restrict__ lam0,
-                                const float *__restrict__ grad, float *__restrict__ out) {
+__global__ void __launch_bounds__(256)
+    k_grad_finalize(const VDom d, const float *__restrict__ lam0, const float *__restrict__ grad,
+                    float *__restrict__ out) {
     using L = Lat<Q>;
-    constexpr int D = L::D;
+    constexpr int D = L::D, A = 1, B = Q == 9 ? 5 : 7;      // an axis and a diagonal direction
     const long long nc = (1 + D) * d.cells;
-    auto G = [&](int comp, long long m) -> double {
-        return (double)grad[comp * d.cells + m] + (double)grad[nc + comp * d.cells + m];
-    };
     for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < d.cells;
          n += (long long)gridDim.x * blockDim.x) {
         int x, y, z;
         cell_xyz(d, n, x, y, z);
         Nb3 Y, Z;
         nb_yz<Q>(d, y, z, Y, Z);
-        double v = G(0, n);
+        TwoFloat sa, sd, la, ld, v;
 #pragma unroll
-        for (int i = 0; i < Q; ++i)
-            v += (double)L::w(i) * (double)lam0[pull_index<Q>(d, i, x, y, z, Y, Z)];
+        for (int i = 1; i < Q; ++i)
+            (i < B ? la : ld).add(lam0[pull_index<Q>(d, i, x, y, z, Y, Z)]);
 #pragma unroll
         for (int i = 1; i < Q; ++i) {
             const int e[3] = {L::ex(i), L::ey(i), L::ez(i)};
+            auto term = [&](long long m) {                  // e_i . G_grad(m)
+#pragma unroll
+                for (int c = 0; c < D; ++c)
+                    if (e[c]) {
+                        const float h = grad[(1 + c) * d.cells + m], l = grad[nc + (1 + c) * d.cells + m];
+                        TwoFloat &s = i < B ? sa : sd;
+                        s.add(e[c] > 0 ? h : -h);
+                        s.add(e[c] > 0 ? l : -l);
+                    }
+            };
             // cell x - e_i, whose stencil reads eps(x) through direction i
             if (!(Y.wall[1 - e[1]] || Z.wall[1 - e[2]])) {
                 int xs = x - e[0];
                 xs = xs < 0 ? xs + d.nx : (xs >= d.nx ? xs - d.nx : xs);
-                const long long m = ((long long)Z.r[1 - e[2]] * d.ny + Y.r[1 - e[1]]) * d.nx + xs;
-                double s = 0.0;
-#pragma unroll
-                for (int c = 0; c < D; ++c) s += e[c] * G(1 + c, m);
-                v += 3.0 * (double)L::w(i) * s;
+                term(((long long)Z.r[1 - e[2]] * d.ny + Y.r[1 - e[1]]) * d.nx + xs);
             }
             // x itself, whose neighbour x + e_i lies past a wall
-            if (Y.wall[1 + e[1]] || Z.wall[1 + e[2]]) {
-                double s = 0.0;
-#pragma unroll
-                for (int c = 0; c < D; ++c) s += e[c] * G(1 + c, n);
-                v += 3.0 * (double)L::w(i) * s;
-            }
+            if (Y.wall[1 + e[1]] || Z.wall[1 + e[2]]) term(n);
         }
-        out[n] = (float)v;
+        TwoFloat l0;
+        l0.h = lam0[pull_index<Q>(d, 0, x, y, z, Y, Z)];
+        v.add(grad[n]);
+        v.add(grad[nc + n]);
+        v.add_scaled(L::w(0), l0);
+        v.add_scaled(L::w(A), la);
+        v.add_scaled(L::w(B), ld);
+        TwoFloat sa3, sd3;                                  // the weights as they are: 3 w would round
+        sa3.add_scaled(3.f, sa);
+        sd3.add_scaled(3.f, sd);
+        v.add_scaled(L::w(A), sa3);
+        v.add_scaled(L::w(B), sd3);
+        out[n] = v.h + v.l;
     }
 }
 
@@ -661,8 +704,8 @@ cudaError_t launch_check(int q, const VDom &d, const float *state, int *flag, cu
 
 cudaError_t launch_flux(int q, const VDom &d, const float *state, int x_out, float *J,
                         cudaStream_t s) {
-    VANS_DISPATCH_Q(q, (k_flux<9><<<1, 256, 0, s>>>(d, state, x_out, J)),
-                    (k_flux<19><<<1, 256, 0, s>>>(d, state, x_out, J)));
+    VANS_DISPATCH_Q(q, (k_flux<9><<<kFluxBlocks, 256, 0, s>>>(d, state, x_out, J)),
+                    (k_flux<19><<<kFluxBlocks, 256, 0, s>>>(d, state, x_out, J)));
     return cudaGetLastError();
 }
 

@@ -1,0 +1,79 @@
+"""The kernels at the two ends of a reverse pass: the outlet flux and the transposed
+grad-eps stencil, against float64 sums of the same numbers."""
+import numpy as np
+import pytest
+
+from paper_1406_6438_gb300 import workloads as W
+from tests._gpu import solver, torch_cuda
+
+pytestmark = pytest.mark.gpu
+
+# (q, (nz, ny, nx)): rows of the outlet plane around the 256 threads and 8 blocks that
+# sum it; axes of one and two cells
+SHAPES = [(9, (1, 1, 5)), (9, (1, 2, 1)), (9, (1, 255, 4)), (9, (1, 2049, 3)), (9, (1, 5000, 2)),
+          (9, (1, 40, 131)), (19, (1, 1, 3)), (19, (2, 3, 2)), (19, (60, 41, 7)), (19, (9, 10, 67))]
+
+
+def _directions(q):
+    r = (-1, 0, 1)
+    if q == 9:
+        w = {0: 4 / 9, 1: 1 / 9, 2: 1 / 36}
+        dirs = [(x, y, 0) for x in r for y in r]
+    else:
+        w = {0: 1 / 3, 1: 1 / 18, 2: 1 / 36}
+        dirs = [(x, y, z) for x in r for y in r for z in r if abs(x) + abs(y) + abs(z) <= 2]
+    return [(e, float(np.float32(w[sum(map(abs, e))]))) for e in dirs]
+
+
+def _case(q, shape, walls, seed):
+    nz, ny, nx = shape
+    p = W.params(q=q, nx=nx, ny=ny, nz=nz, wall_mask=walls, tau=0.7, g=(3e-4, 0.0, 0.0),
+                 drag_mode=2, k_mode=0, d_p=6.0)
+    eps = W.smoothed_noise(shape, 2.0, 0.4, 1.0, seed)
+    return p, eps, W.random_state(q, eps, seed + 1, amp=0.02)
+
+
+@pytest.mark.parametrize("q,shape", SHAPES)
+def test_flux_is_the_sum_of_the_outlet(q, shape):
+    """Tolerance: eps, rho and u carry an fp32 rounding or two each, relative to the
+    cells' magnitudes (the sum itself cancels)."""
+    torch = torch_cuda()
+    p, eps, f0 = _case(q, shape, 2, seed=sum(shape))
+    s = solver(p, eps)
+    s.set_populations(torch.from_numpy(f0).cuda())
+    J = float(s.flux(shape[2] - 1))
+    rho, u = s.moments()
+    terms = (eps.reshape(shape).astype(np.float64) * rho.cpu().numpy().reshape(shape) *
+             u[0].cpu().numpy().reshape(shape))[:, :, -1]
+    assert abs(J - terms.sum()) <= 1e-6 * np.abs(terms).sum()
+
+
+@pytest.mark.parametrize("walls", [0, 2, 6])
+@pytest.mark.parametrize("q,shape", SHAPES)
+def test_gradient_stencil(q, shape, walls):
+    """lambda = 0, accumulators of 1e4 whose stencil cancels to a difference: to the
+    rounding of the result, and 2^-42 of the terms for the two-float sums of 36."""
+    torch = torch_cuda()
+    if q == 9 and walls == 6:
+        pytest.skip("no z walls in two dimensions")
+    nz, ny, nx = shape
+    D = 2 if q == 9 else 3
+    p, eps, _ = _case(q, shape, walls, seed=2)
+    s = solver(p, eps)
+    rng = np.random.default_rng(5)
+    head = (1e4 + rng.standard_normal((1 + D,) + shape)).astype(np.float32)
+    head[0] = rng.standard_normal(shape)
+    tail = (1e-4 * rng.standard_normal((1 + D,) + shape)).astype(np.float32)
+    acc = torch.from_numpy(np.concatenate([head.ravel(), tail.ravel()])).cuda()
+    out = s.grad_finalize(s.new_state(), acc).cpu().numpy().reshape(shape)
+    G = head.astype(np.float64) + tail
+    v = G[0].copy()
+    z, y, x = np.meshgrid(*(np.arange(n) for n in shape), indexing="ij")
+    for e, w in _directions(q):
+        def past(sign):
+            yy, zz = y + sign * e[1], z + sign * e[2]
+            return ((walls & 2 != 0) & ((yy < 0) | (yy >= ny))) | ((walls & 4 != 0) & ((zz < 0) | (zz >= nz)))
+        src = G[:, (z - e[2]) % nz, (y - e[1]) % ny, (x - e[0]) % nx]
+        for field, where in ((src, ~past(-1)), (G, past(1))):
+            v += np.where(where, 3 * w * sum(e[c] * field[1 + c] for c in range(D)), 0.0)
+    assert np.all(np.abs(out - v) <= 2.0 ** -23 * np.abs(v) + 2.0 ** -42 * 1e4 * 36)
