@@ -175,6 +175,8 @@ struct vans_s {
     cudaGraphExec_t gexec[kGraphSizes] = {};   // 64, 32, ..., 2 single-step launches
     cudaGraphExec_t gmulti[kGraphSizes] = {};  // as many kind 9 launches of L.rows steps
     int *flag = nullptr;                        // device status words (workspace)
+    int *flag_host = nullptr;                   // pinned copy of flag[0] (vans_update_eps)
+    cudaEvent_t flag_read = nullptr;            // behind that copy
     float *mon_part = nullptr;                  // monitoring partial maxima (workspace)
     int adj_fp64 = 0;                           // reverse-step arithmetic in FP64
     Launch adjL{1, 4, 4, 1};                    // reverse-step launch shape
@@ -352,6 +354,20 @@ int make_streams(vans_t h, void *stream) {
     if (cudaGetDevice(&h->device) != cudaSuccess) return VANS_ERR_CUDA;
     if (cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking) != cudaSuccess) return VANS_ERR_CUDA;
     return VANS_OK;
+}
+
+// the pinned word and the event of vans_update_eps, made when it is first called.
+// Allocating and freeing pinned memory is allowed whatever another thread captures.
+int host_flag(vans_t h) {
+    if (h->flag_host) return VANS_OK;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    cudaError_t e = cudaSuccess;
+    if (!h->flag_read) e = cudaEventCreateWithFlags(&h->flag_read, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaHostAlloc((void **)&h->flag_host, sizeof(int), cudaHostAllocDefault);
+    if (e != cudaSuccess) h->flag_host = nullptr;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return cuda_status(e);
 }
 
 // read the status words (flag[0]: range / divergence, flag[1]: a bounded
@@ -648,6 +664,13 @@ void vans_destroy(vans_t h) {
     if (!h) return;
     drop_graph(h);
     if (h->cap) cudaStreamDestroy(h->cap);
+    if (h->flag_read) cudaEventDestroy(h->flag_read);
+    if (h->flag_host) {
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        cudaFreeHost(h->flag_host);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+    }
     delete h;
 }
 
@@ -655,7 +678,7 @@ int vans_set_eps(vans_t h, const float *eps_dev) {
     if (!h || h->batched || !eps_dev) return VANS_ERR_ARG;
     if (cudaMemsetAsync(h->flag, 0, sizeof(int), h->stream) != cudaSuccess) return VANS_ERR_CUDA;
     ++h->launches;
-    if (vans::launch_pad_eps(h->dom, eps_dev, nullptr, h->flag, h->stream) != cudaSuccess)
+    if (vans::launch_check_eps(h->dom, eps_dev, h->flag, h->stream) != cudaSuccess)
         return VANS_ERR_CUDA;
     int bad = 0;
     int rc = read_flag(h, &bad);
@@ -682,20 +705,21 @@ int vans_update_eps(vans_t h, const float *eps_dev) {
     if (!h || h->batched || !eps_dev) return VANS_ERR_ARG;
     if (!h->eps_set) return VANS_ERR_STATE;
     if (h->slab) return VANS_ERR_UNSUPPORTED;
+    if (const int rc = host_flag(h)) return rc;
     if (cudaMemsetAsync(h->flag, 0, sizeof(int), h->stream) != cudaSuccess) return VANS_ERR_CUDA;
-    ++h->launches;
-    if (vans::launch_pad_eps(h->dom, eps_dev, nullptr, h->flag, h->stream) != cudaSuccess)
+    h->launches += 3;
+    // the update is enqueued before the flag is read here, and held back by it on the
+    // device: the stream does not run dry while the host waits for the flag and returns
+    // to enqueue steps (1536 x 1000: 24 us per update)
+    if (vans::launch_check_eps(h->dom, eps_dev, h->flag, h->stream) != cudaSuccess ||
+        cudaMemcpyAsync(h->flag_host, h->flag, sizeof(int), cudaMemcpyDeviceToHost, h->stream) !=
+            cudaSuccess ||
+        cudaEventRecord(h->flag_read, h->stream) != cudaSuccess ||
+        vans::launch_rebase_eps(h->q, h->dom, eps_dev, h->st[h->cur], h->flag, h->stream) != cudaSuccess ||
+        vans::launch_pad_eps(h->dom, eps_dev, h->eps_pad, h->flag + 3, h->stream, h->flag) != cudaSuccess ||
+        cudaEventSynchronize(h->flag_read) != cudaSuccess)
         return VANS_ERR_CUDA;
-    int bad = 0;
-    int rc = read_flag(h, &bad);
-    if (rc) return rc;
-    if (bad) return VANS_ERR_ARG;
-    h->launches += 2;
-    if (vans::launch_rebase_eps(h->q, h->dom, eps_dev, h->st[h->cur], h->stream) != cudaSuccess)
-        return VANS_ERR_CUDA;
-    if (vans::launch_pad_eps(h->dom, eps_dev, h->eps_pad, h->flag, h->stream) != cudaSuccess)
-        return VANS_ERR_CUDA;
-    return VANS_OK;
+    return *h->flag_host ? VANS_ERR_ARG : VANS_OK;
 }
 
 int vans_step(vans_t h, int nsteps) {
@@ -721,22 +745,29 @@ int vans_step_monitored(vans_t h, int nsteps, int every, float *rho_dev, float *
     if (cudaMemsetAsync(stats_dev, 0, 4 * sizeof(float), h->stream) != cudaSuccess ||
         cudaMemsetAsync(h->mon_part, 0, kMonFloats * sizeof(float), h->stream) != cudaSuccess)
         return VANS_ERR_CUDA;
-    int done = 0;
+    // An emission reads the state before the step that it stands for.  With several
+    // steps per launch that step goes with the plain ones up to the next emission
+    // (2048^2: 62 us for the emission and 27 for the step, in one kernel 111); single
+    // steps emit themselves (4096^2: 420 us, 215 + 250 apart).
+    const bool fused = h->L.kind != 9 || every == 1;
+    int done = 0, owed = 0;
     while (done < nsteps) {
-        // every-1 plain steps (graph-replayed when long), then one monitoring step
         const int plain = std::min(every - 1, nsteps - done - 1);
-        if (plain > 0) {
-            const int rc = run_steps(h, plain);
-            if (rc) return rc;
-            done += plain;
-        }
+        const int rc = run_steps(h, owed + plain);
+        if (rc) return rc;
+        done += plain + 1;
         ++h->launches;
-        if (vans::launch_step_monitor(h->q, h->dom, h->st[h->cur], h->st[h->cur ^ 1], rho_dev, u_dev,
-                                      stats_dev, h->mon_part, h->stream) != cudaSuccess)
+        const float *in = h->st[h->cur];
+        if ((fused ? vans::launch_step_monitor(h->q, h->dom, in, h->st[h->cur ^ 1], rho_dev, u_dev, stats_dev,
+                                               h->mon_part, h->stream)
+                   : vans::launch_moments_rows(h->dom, in, rho_dev, u_dev, stats_dev, h->mon_part,
+                                               h->stream)) != cudaSuccess)
             return VANS_ERR_CUDA;
-        h->cur ^= 1;
-        ++done;
+        if (fused) h->cur ^= 1;
+        else owed = 1;
     }
+    const int rc = run_steps(h, owed);
+    if (rc) return rc;
     if (nsteps > 0) {
         ++h->launches;
         if (vans::launch_monitor_finalize(h->mon_part, stats_dev, h->stream) != cudaSuccess)
@@ -1200,7 +1231,7 @@ int vans_batch_set_eps(vans_t h, int d, const float *eps_dev) {
     const VDom &D = h->doms[d];
     if (cudaMemsetAsync(h->flag, 0, sizeof(int), h->stream) != cudaSuccess) return VANS_ERR_CUDA;
     ++h->launches;
-    if (vans::launch_pad_eps(D, eps_dev, nullptr, h->flag, h->stream) != cudaSuccess)
+    if (vans::launch_check_eps(D, eps_dev, h->flag, h->stream) != cudaSuccess)
         return VANS_ERR_CUDA;
     int bad = 0;
     int rc = read_flag(h, &bad);

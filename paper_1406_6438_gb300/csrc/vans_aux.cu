@@ -200,10 +200,13 @@ __global__ void k_init_moving(const VDom d, float *__restrict__ st) {
 // stores f - w eps~ (minus the moving-wall gain where one applies), so it is
 // re-expressed from the old eps (the padded rows still in d.eps) to the new
 // one (dense eps_new).  Each entry belongs to exactly one cell (pull_index is
-// a bijection), so the update runs in place.
+// a bijection), so the update runs in place.  Nothing is written where the check
+// before it flagged eps_new.
 template <int Q>
-__global__ void k_rebase_eps(const VDom d, const float *__restrict__ eps_new, float *__restrict__ st) {
+__global__ void k_rebase_eps(const VDom d, const float *__restrict__ eps_new, float *__restrict__ st,
+                             const int *__restrict__ flag) {
     using L = Lat<Q>;
+    const int refused = *flag;            // (looked at after the loads)
     for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < d.cells;
          n += (long long)gridDim.x * blockDim.x) {
         int x, y, z;
@@ -218,6 +221,7 @@ __global__ void k_rebase_eps(const VDom d, const float *__restrict__ eps_new, fl
         float v[Q];
 #pragma unroll
         for (int i = 0; i < Q; ++i) v[i] = st[pull_index<Q>(d, i, x, y, z, Y, Z)];
+        if (refused) return;
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             v[i] += L::w(i) * (e_old - e_new);
@@ -228,37 +232,58 @@ __global__ void k_rebase_eps(const VDom d, const float *__restrict__ eps_new, fl
     }
 }
 
-// eps into padded rows with periodic halo columns; padding gets 1.0.  Flags any
-// value outside (0, 1] (NaN included).
+// Flags any porosity outside (0, 1] (NaN included).
+__global__ void k_check_eps(long long n, const float *__restrict__ eps, bool vec, int *flag) {
+    const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long step = (long long)gridDim.x * blockDim.x;
+    bool bad = false;
+    auto test = [&](float v) { bad = bad || !(v > 0.0f && v <= 1.0f); };
+    if (vec) {
+        for (long long t = t0; t < n / 4; t += step) {
+            const float4 v = __ldg(reinterpret_cast<const float4 *>(eps) + t);
+            test(v.x);
+            test(v.y);
+            test(v.z);
+            test(v.w);
+        }
+    }
+    for (long long t = t0 + (vec ? n / 4 * 4 : 0); t < n; t += step) test(eps[t]);
+    if (bad) atomicOr(flag, 1);
+}
+
+// eps into padded rows with periodic halo columns; padding gets 1.0.  Flags as
+// k_check_eps does.  A thread writes four columns (pitch and off are multiples of 4):
+// with one, its division by the pitch took more than its bytes (1536 x 1000 9.9 us, now
+// 6.0).  held (nullptr: none): a flag that, set, leaves pad as it is.
 __global__ void k_pad_eps(const VDom d, const float *__restrict__ eps, float *__restrict__ pad,
-                          int *flag) {
-    const long long total = (long long)d.rows * d.pitch;
+                          int *flag, const int *__restrict__ held) {
+    if (held && *held) return;
+    const unsigned quads = (unsigned)d.pitch / 4;
+    const long long total = (long long)d.rows * quads;
+    bool bad = false;
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
          t += (long long)gridDim.x * blockDim.x) {
-        long long r;
-        int c;
-        if (total <= 0xffffffffLL) {            // 32-bit division where it suffices
-            const unsigned tt = (unsigned)t, rr = tt / (unsigned)d.pitch;
-            r = rr;
-            c = (int)(tt - rr * (unsigned)d.pitch) - d.off;
-        } else {
-            r = t / d.pitch;
-            c = (int)(t % d.pitch) - d.off;
+        // 32-bit division where it suffices
+        const long long r = total <= 0xffffffffLL ? (long long)((unsigned)t / quads) : t / quads;
+        const int c0 = (int)(t - r * quads) * 4 - d.off;
+        const float *row = eps + r * d.nx;
+        float v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int c = c0 + k;
+            v[k] = 1.0f;
+            if (c >= 0 && c < d.nx) {
+                v[k] = __ldg(row + c);
+                bad = bad || !(v[k] > 0.0f && v[k] <= 1.0f);
+            } else if (c == -1) {
+                v[k] = __ldg(row + d.nx - 1);
+            } else if (c == d.nx) {
+                v[k] = __ldg(row);
+            }
         }
-        float v = 1.0f;
-        if (c >= 0 && c < d.nx) {
-            v = eps[r * d.nx + c];
-            if (!(v > 0.0f && v <= 1.0f)) atomicOr(flag, 1);
-            if (pad == nullptr) continue;       // range check only
-        } else if (pad == nullptr) {
-            continue;
-        } else if (c == -1) {
-            v = eps[r * d.nx + d.nx - 1];
-        } else if (c == d.nx) {
-            v = eps[r * d.nx];
-        }
-        pad[t] = v;
+        reinterpret_cast<float4 *>(pad)[t] = make_float4(v[0], v[1], v[2], v[3]);
     }
+    if (bad) atomicOr(flag, 1);
 }
 
 template <int Q>
@@ -652,6 +677,7 @@ static int grid_for(long long n, int threads) {
 
 cudaError_t launch_moments(int q, const VDom &d, const float *state, float *rho, float *u,
                            cudaStream_t s) {
+    if (q == 9 && !d.nee) return launch_moments_rows(d, state, rho, u, nullptr, nullptr, s);
     const int g = grid_for(d.cells, 256);
     VANS_DISPATCH_Q(q, (k_moments<9><<<g, 256, 0, s>>>(d, state, rho, u)),
                     (k_moments<19><<<g, 256, 0, s>>>(d, state, rho, u)));
@@ -673,17 +699,23 @@ cudaError_t launch_import(int q, const VDom &d, const float *f, float *state, cu
 }
 
 cudaError_t launch_pad_eps(const VDom &d, const float *eps_dense, float *eps_pad, int *flag,
-                           cudaStream_t s) {
-    const int g = grid_for((long long)d.rows * d.pitch, 256);
-    k_pad_eps<<<g, 256, 0, s>>>(d, eps_dense, eps_pad, flag);
+                           cudaStream_t s, const int *held) {
+    const int g = grid_for((long long)d.rows * (d.pitch / 4), 256);
+    k_pad_eps<<<g, 256, 0, s>>>(d, eps_dense, eps_pad, flag, held);
     return cudaGetLastError();
 }
 
-cudaError_t launch_rebase_eps(int q, const VDom &d, const float *eps_new, float *state,
+cudaError_t launch_check_eps(const VDom &d, const float *eps_dense, int *flag, cudaStream_t s) {
+    const bool vec = ((uintptr_t)eps_dense & 15) == 0;
+    k_check_eps<<<grid_for(vec ? (d.cells + 3) / 4 : d.cells, 256), 256, 0, s>>>(d.cells, eps_dense, vec, flag);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_rebase_eps(int q, const VDom &d, const float *eps_new, float *state, const int *flag,
                               cudaStream_t s) {
     const int g = grid_for(d.cells, 256);
-    VANS_DISPATCH_Q(q, (k_rebase_eps<9><<<g, 256, 0, s>>>(d, eps_new, state)),
-                    (k_rebase_eps<19><<<g, 256, 0, s>>>(d, eps_new, state)));
+    VANS_DISPATCH_Q(q, (k_rebase_eps<9><<<g, 256, 0, s>>>(d, eps_new, state, flag)),
+                    (k_rebase_eps<19><<<g, 256, 0, s>>>(d, eps_new, state, flag)));
     return cudaGetLastError();
 }
 

@@ -80,6 +80,7 @@ cudaError_t launch_step(int q, const VDom &d, const float *fin, float *fout, Lau
                         cudaStream_t stream);
 // partial maxima of the monitoring reductions: kMonSlots per statistic
 constexpr int kMonSlots = 256;
+// a step that emits too
 cudaError_t launch_step_monitor(int q, const VDom &d, const float *fin, float *fout, float *rho,
                                 float *u, float *stats, float *part, cudaStream_t stream);
 // stats[0..2] = maxima of the partials (after the monitoring steps of a call)
@@ -118,11 +119,17 @@ cudaError_t launch_step_batched(const VDom *doms_dev, const Tile *tiles_dev, int
 int batched_blocks_per_sm(Launch L);
 cudaError_t launch_moments(int q, const VDom &d, const float *state, float *rho, float *u,
                            cudaStream_t stream);
+// launch_moments for D2Q9 without plates on nodes; with stats the reductions of a
+// monitoring emission too (u: the previous emission's on entry)
+cudaError_t launch_moments_rows(const VDom &d, const float *state, float *rho, float *u,
+                                float *stats, float *part, cudaStream_t stream);
 cudaError_t launch_export(int q, const VDom &d, const float *state, float *f, cudaStream_t stream);
 cudaError_t launch_import(int q, const VDom &d, const float *f, float *state, cudaStream_t stream);
 cudaError_t launch_pad_eps(const VDom &d, const float *eps_dense, float *eps_pad, int *flag,
-                           cudaStream_t stream);
-cudaError_t launch_rebase_eps(int q, const VDom &d, const float *eps_new, float *state,
+                           cudaStream_t stream, const int *held = nullptr);
+cudaError_t launch_check_eps(const VDom &d, const float *eps_dense, int *flag, cudaStream_t stream);
+// the state under a new porosity (d.eps: the old one), unless *flag is set
+cudaError_t launch_rebase_eps(int q, const VDom &d, const float *eps_new, float *state, const int *flag,
                               cudaStream_t stream);
 cudaError_t launch_init_moving(int q, const VDom &d, float *state, cudaStream_t stream);
 cudaError_t launch_check(int q, const VDom &d, const float *state, int *flag, cudaStream_t stream);

@@ -11,6 +11,8 @@
 // D2Q9, a (y,z) line for D3Q19); each lane owns CPT cells and loads them with
 // one aligned vector load per direction.  The +-1 column shift of the pull is
 // done with a warp shuffle, so every global load is an aligned vector load.
+#include <algorithm>
+
 #include "vans_device.cuh"
 
 namespace vans {
@@ -28,6 +30,65 @@ struct Monitor {
 __device__ __forceinline__ void atomic_max_nonneg(float *a, float v) {
     // non-negative floats order like their bit patterns
     atomicMax(reinterpret_cast<int *>(a), __float_as_int(v));
+}
+
+// The maxima of a warp into the partial maxima of an emission.
+__device__ __forceinline__ void emit_maxima(const Monitor &mon, int lane, float dmax, float umax, bool bad) {
+            // warp maxima, one atomic per warp
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                dmax = fmaxf(dmax, __shfl_xor_sync(VANS_FULL, dmax, off));
+                umax = fmaxf(umax, __shfl_xor_sync(VANS_FULL, umax, off));
+            }
+            bad = __any_sync(VANS_FULL, bad);
+            if (lane == 0) {
+                // one of kMonSlots partial maxima per warp: with every warp on the
+                // same three words the step took 634 us at 4096^2, 420 us spread
+                const int slot = (int)((blockIdx.x * ((blockDim.x * blockDim.y) >> 5) +
+                                        ((threadIdx.y * blockDim.x + threadIdx.x) >> 5)) &
+                                       (kMonSlots - 1));
+                atomic_max_nonneg(&mon.part[slot], bad ? 0.f : dmax);
+                atomic_max_nonneg(&mon.part[kMonSlots + slot], bad ? 0.f : umax);
+                if (bad) atomic_max_nonneg(&mon.part[2 * kMonSlots + slot], 1.f);
+            }
+}
+
+// What the update of CPT cells from x0 on in row (y, z) reads: the pulled populations h
+// and the porosities E[1 + dy][1 + dz][1 + k + dx] (D3Q19 corner rows at dx = 0 only).
+template <int Q, int CPT>
+__device__ __forceinline__ void load_row(const VDom &d, const float *__restrict__ fin, const Nb3 &Y,
+                                         const Nb3 &Z, int y, int z, int x0, int lane, float h[Q][CPT],
+                                         float E[3][3][CPT + 2]) {
+    using L = Lat<Q>;
+    // S1: pull.  h_i(x) = stored deviation at x - e_i, or the opposite
+    // direction of x itself when x - e_i lies past a wall.
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const int ex = L::ex(i), ey = L::ey(i), ez = L::ez(i);
+        const bool bb = Y.wall[1 - ey] || Z.wall[1 - ez];
+        const int si = bb ? L::opp(i) : i;
+        const long long ro = bb ? row_offset(d, y, z) : row_offset(d, Y.r[1 - ey], Z.r[1 - ez]);
+        ld_shift<CPT>(fin + si * d.plane + ro, x0, bb ? 0 : -ex, lane, h[i]);
+    }
+
+    // porosity of the cell and of its Q-1 neighbours (for grad eps and the
+    // deviation shift), from the padded eps rows
+#pragma unroll
+    for (int dz = -1; dz <= 1; ++dz) {
+#pragma unroll
+        for (int dy = -1; dy <= 1; ++dy) {
+            if (Q == 9 && dz != 0) continue;
+            const float *row = d.eps + row_offset(d, Y.r[1 + dy], Z.r[1 + dz]);
+            if (dy != 0 && dz != 0) {
+                float t[CPT];
+                ld_vec<CPT>(row + x0, t);
+#pragma unroll
+                for (int k = 0; k < CPT; ++k) E[1 + dy][1 + dz][k + 1] = t[k];
+            } else {
+                ld_ext<CPT>(row, x0, lane, E[1 + dy][1 + dz]);
+            }
+        }
+    }
 }
 
 // PL: the instance handles plates on nodes (wall_kind 1); the others carry
@@ -50,37 +111,8 @@ __device__ __forceinline__ void step_row(const VDom &d, const float *__restrict_
         Z.wall[0] = Z.wall[1] = Z.wall[2] = false;
     }
 
-    // S1: pull.  h_i(x) = stored deviation at x - e_i, or the opposite
-    // direction of x itself when x - e_i lies past a wall.
-    float h[Q][CPT];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const int ex = L::ex(i), ey = L::ey(i), ez = L::ez(i);
-        const bool bb = Y.wall[1 - ey] || Z.wall[1 - ez];
-        const int si = bb ? L::opp(i) : i;
-        const long long ro = bb ? row_offset(d, y, z) : row_offset(d, Y.r[1 - ey], Z.r[1 - ez]);
-        ld_shift<CPT>(fin + si * d.plane + ro, x0, bb ? 0 : -ex, lane, h[i]);
-    }
-
-    // porosity of the cell and of its Q-1 neighbours (for grad eps and the
-    // deviation shift), from the padded eps rows
-    float E[3][3][CPT + 2];
-#pragma unroll
-    for (int dz = -1; dz <= 1; ++dz) {
-#pragma unroll
-        for (int dy = -1; dy <= 1; ++dy) {
-            if (Q == 9 && dz != 0) continue;
-            const float *row = d.eps + row_offset(d, Y.r[1 + dy], Z.r[1 + dz]);
-            if (dy != 0 && dz != 0) {
-                float t[CPT];
-                ld_vec<CPT>(row + x0, t);
-#pragma unroll
-                for (int k = 0; k < CPT; ++k) E[1 + dy][1 + dz][k + 1] = t[k];
-            } else {
-                ld_ext<CPT>(row, x0, lane, E[1 + dy][1 + dz]);
-            }
-        }
-    }
+    float h[Q][CPT], E[3][3][CPT + 2];
+    load_row<Q, CPT>(d, fin, Y, Z, y, z, x0, lane, h, E);
 
     // the monitored step's previous u, loaded with the populations: read after
     // this thread's first moment stores, the loads (which may alias them) were
@@ -146,25 +178,7 @@ __device__ __forceinline__ void step_row(const VDom &d, const float *__restrict_
             }
         }
     }
-    if (EMIT) {
-        // warp maxima, one atomic per warp
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            dmax = fmaxf(dmax, __shfl_xor_sync(VANS_FULL, dmax, off));
-            umax = fmaxf(umax, __shfl_xor_sync(VANS_FULL, umax, off));
-        }
-        bad = __any_sync(VANS_FULL, bad);
-        if (lane == 0) {
-            // one of kMonSlots partial maxima per warp: with every warp on the
-            // same three words the step took 634 us at 4096^2, 420 us spread
-            const int slot = (int)((blockIdx.x * ((blockDim.x * blockDim.y) >> 5) +
-                                    ((threadIdx.y * blockDim.x + threadIdx.x) >> 5)) &
-                                   (kMonSlots - 1));
-            atomic_max_nonneg(&mon->part[slot], bad ? 0.f : dmax);
-            atomic_max_nonneg(&mon->part[kMonSlots + slot], bad ? 0.f : umax);
-            if (bad) atomic_max_nonneg(&mon->part[2 * kMonSlots + slot], 1.f);
-        }
-    }
+    if (EMIT) emit_maxima(*mon, lane, dmax, umax, bad);
 
     const long long ro = row_offset(d, y, z);
 #pragma unroll
@@ -208,6 +222,108 @@ __global__ void __launch_bounds__(256) k_step(const VDom d, const float *__restr
         step_row<Q, CPT, true, EMIT, PL>(d, fin, fout, y, z, x0, lane, &mon);
     else
         step_row<Q, CPT, false, EMIT, PL>(d, fin, fout, y, z, x0, lane, &mon);
+    if (EMIT && blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) atomicAdd(&mon.stats[3], 1.f);
+}
+
+template <int Q, int CPT, bool EDGE, bool EMIT>
+__device__ __forceinline__ void moments_row(const VDom &d, const float *__restrict__ fin, const Monitor &mon,
+                                            bool whole, int y, int z, int x0, int lane) {
+    using L = Lat<Q>;
+    const Nb3 Y = nb3<EDGE>(y, d.ny, d.wall_y);
+    Nb3 Z;
+    if (Q == 19) {
+        Z = nb3<EDGE>(z, d.nz, d.wall_z);
+    } else {
+        Z.r[0] = Z.r[1] = Z.r[2] = 0;
+        Z.wall[0] = Z.wall[1] = Z.wall[2] = false;
+    }
+    float h[Q][CPT], E[3][3][CPT + 2];
+    load_row<Q, CPT>(d, fin, Y, Z, y, z, x0, lane, h, E);
+    const long long n = ((long long)z * d.ny + y) * d.nx + x0;
+    // whole: every row of the dense outputs starts on a vector boundary
+    auto put = [&](float *p, const float v[CPT]) {
+        if (whole && x0 + CPT <= d.nx) {
+            st_vec<CPT>(p + n, v);
+        } else {
+#pragma unroll
+            for (int k = 0; k < CPT; ++k)
+                if (x0 + k < d.nx) p[n + k] = v[k];
+        }
+    };
+    float up[L::D][CPT];
+    if (EMIT) {
+#pragma unroll
+        for (int c = 0; c < L::D; ++c) {
+            const float *p = mon.u + c * d.cells + n;
+            if (whole && x0 + CPT <= d.nx) {
+                struct alignas(4 * CPT) Cells { float v[CPT]; };
+                const Cells t = *reinterpret_cast<const Cells *>(p);     // (written below: not ld_vec)
+#pragma unroll
+                for (int k = 0; k < CPT; ++k) up[c][k] = t.v[k];
+            } else {
+#pragma unroll
+                for (int k = 0; k < CPT; ++k) up[c][k] = x0 + k < d.nx ? p[k] : 0.f;
+            }
+        }
+    }
+    float rho[CPT], u[L::D][CPT], dmax = 0.f, umax = 0.f;
+    bool bad = false;
+#pragma unroll
+    for (int k = 0; k < CPT; ++k) {
+        float hh[Q], et[Q];
+        const float e0 = E[1][1][k + 1];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            hh[i] = h[i][k];
+            const bool wall = Y.wall[1 + L::ey(i)] || Z.wall[1 + L::ez(i)];
+            et[i] = (i == 0 || wall) ? e0 : E[1 + L::ey(i)][1 + L::ez(i)][k + 1 + L::ex(i)];
+        }
+        if (EDGE) apply_moving_wall<Q>(d, Y.wall[2], Z, e0, hh);
+        Macro<Q> M;
+        macro<Q>(d, hh, e0, et, M);
+        rho[k] = M.rho;
+        float du2 = 0.f;
+#pragma unroll
+        for (int c = 0; c < L::D; ++c) {
+            u[c][k] = M.u[c];
+            if (EMIT) du2 += (M.u[c] - up[c][k]) * (M.u[c] - up[c][k]);
+        }
+        if (EMIT && x0 + k < d.nx) {
+            dmax = fmaxf(dmax, sqrtf(du2));
+            umax = fmaxf(umax, M.un);
+            bad = bad || !isfinite(M.R) || !isfinite(M.un) || !(M.un < 0.5f);
+        }
+    }
+    if (mon.rho) put(mon.rho, rho);
+    if (mon.u) {
+#pragma unroll
+        for (int c = 0; c < L::D; ++c) put(mon.u + c * d.cells, u[c]);
+    }
+    if (EMIT) emit_maxima(mon, lane, dmax, umax, bad);
+}
+
+// rho and u of the state (Eqs. 0moment and 1moment), and with EMIT the reductions of
+// a monitoring emission.  Bound by the loads in flight: rows by vector loads (4 cells
+// per lane) with as many blocks per SM as the registers allow without spills, 7 (6 with
+// EMIT): 4096^2 245 -> 158 us (0.82 of the copy bandwidth), 2048^2 68 -> 47, 1501 x 733
+// 20.4 -> 13.1, against one cell per thread.  D3Q19 keeps that form (vans_aux.cu): 2
+// cells per lane measured the same at 256 x 256 x 128 and 64 us instead of 48 at
+// 150 x 110 x 90.
+template <int Q, int CPT, bool EMIT>
+__global__ void __launch_bounds__(128, EMIT ? 6 : 7) k_moments_rows(const VDom d, const float *__restrict__ fin, int nxb,
+                                                      const Monitor mon, bool whole) {
+    pdl_trigger();
+    pdl_wait();
+    const int lane = threadIdx.x & 31, wx = threadIdx.x >> 5;
+    const int bx = blockIdx.x % nxb, r = (blockIdx.x / nxb) * blockDim.y + threadIdx.y;
+    const int xw = (bx * (blockDim.x >> 5) + wx) * 32 * CPT;
+    if (r >= d.rows || xw >= d.nx) return;                 // whole warp
+    const int y = r % d.ny, z = r / d.ny;
+    const bool edge = (y == 0) || (y == d.ny - 1) || (Q == 19 && (z == 0 || z == d.nz - 1));
+    if (edge)
+        moments_row<Q, CPT, true, EMIT>(d, fin, mon, whole, y, z, xw + lane * CPT, lane);
+    else
+        moments_row<Q, CPT, false, EMIT>(d, fin, mon, whole, y, z, xw + lane * CPT, lane);
     if (EMIT && blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) atomicAdd(&mon.stats[3], 1.f);
 }
 
@@ -289,6 +405,26 @@ cudaError_t launch_step_monitor(int q, const VDom &d, const float *fin, float *f
     else
         return cudaErrorInvalidValue;
     return cudaGetLastError();
+}
+
+template <int Q, int CPT, bool EMIT>
+static cudaError_t launch_moments_t(const VDom &d, const float *state, const Monitor &mon,
+                                    cudaStream_t stream) {
+    const int warps = std::min(4, (d.nx + 32 * CPT - 1) / (32 * CPT)), rows = 4 / warps;
+    const int nxb = (d.nx + 32 * CPT * warps - 1) / (32 * CPT * warps);
+    const long long nblocks = (long long)nxb * ((d.rows + rows - 1) / rows);
+    if (nblocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    const bool whole = d.nx % CPT == 0 && ((uintptr_t)mon.rho | (uintptr_t)mon.u) % (4 * CPT) == 0;
+    return launch_pdl(k_moments_rows<Q, CPT, EMIT>, dim3((unsigned)nblocks), dim3(32 * warps, rows), 0, stream,
+                      d, state, nxb, mon, whole);
+}
+
+cudaError_t launch_moments_rows(const VDom &d, const float *state, float *rho, float *u,
+                                float *stats, float *part, cudaStream_t stream) {
+    const Monitor mon{rho, u, stats, part};
+    if (d.q != 9) return cudaErrorInvalidValue;
+    return stats ? launch_moments_t<9, 4, true>(d, state, mon, stream)
+                 : launch_moments_t<9, 4, false>(d, state, mon, stream);
 }
 
 // stats[c] = max over the slots of part[c][slot], c = 0..2 (one block)
