@@ -17,6 +17,10 @@
 // releases a stage as soon as it has read it into registers.  The accumulator
 // words of a tile are loaded before the tile's wait, so their latency hides
 // behind it.
+//
+// Bound by its arithmetic's latency (D3Q19: 128 registers, 9 to 14 warps per SM):
+// what counts is that those warps' lanes hold cells, so D3Q19 takes the tile width
+// that fits the rows (vans_create).
 #include "vans_adjoint.cuh"
 #include "vans_pipeline.cuh"
 
@@ -245,7 +249,7 @@ static cudaError_t launch_adj_tma_t(const VDom &d, const float *state, const flo
     return cudaGetLastError();
 }
 
-// L.warps -> compute warps (2 or 4), L.cpt -> cells per thread per tile (D2Q9
+// L.warps -> compute warps (2 or 4, D3Q19 2 to 7), L.cpt -> cells per thread per tile (D2Q9
 // 1 or 2, D3Q19 1), L.rows -> pipeline stages
 cudaError_t launch_adjoint_tma(int q, const VDom &d, const float *state, const float *lam_in,
                                float *lam_out, float *grad, int fp64, Launch L, cudaStream_t s) {
@@ -257,7 +261,12 @@ cudaError_t launch_adjoint_tma(int q, const VDom &d, const float *state, const f
     VANS_ADJ_CASE(9, 64, 1)
     VANS_ADJ_CASE(9, 128, 1)
     VANS_ADJ_CASE(9, 128, 2)
+    VANS_ADJ_CASE(19, 64, 1)
+    VANS_ADJ_CASE(19, 96, 1)
     VANS_ADJ_CASE(19, 128, 1)
+    VANS_ADJ_CASE(19, 160, 1)
+    VANS_ADJ_CASE(19, 192, 1)
+    VANS_ADJ_CASE(19, 224, 1)
 #undef VANS_ADJ_CASE
     return cudaErrorInvalidValue;
 }

@@ -645,7 +645,15 @@ int vans_create(const vans_params *p, void *workspace, size_t workspace_bytes, v
     h->L = h->Ls = single_default(p->q);
     // the pipelined reverse step, one cell per thread, 4 stages: fastest on GB300 at 512^2
     // (backward pass 17.4 us per step against 20.8 with the register-load kernel)
-    h->adjL = (p->q == 19) ? Launch{1, 4, 2, 1} : Launch{1, 4, 4, 1};   // D3Q19: 0.78 vs 0.61 of HBM
+    h->adjL = Launch{1, 4, 4, 1};
+    if (p->q == 19) {
+        // tiles of 64 to 224 cells, the narrowest that take a row in as few as there can
+        // be: with 128 cells whatever the row, 150 x 110 x 90 took 148 us per reverse step
+        // (160 cells 97, 192 101, 224 118), 96 x 64 x 48 30 (96 cells 24), 64^3 33 (26),
+        // 222 x 80 x 80 99 (83); 128- and 256-cell rows keep it (73 and 65 us, others 86+)
+        const int tiles = (p->nx + 223) / 224, cells = (p->nx + tiles - 1) / tiles;
+        h->adjL = Launch{1, std::max(2, (cells + 31) / 32), 2, 1};
+    }
     int rc = make_streams(h, cuda_stream);
     if (rc) {
         vans_destroy(h);
@@ -1023,10 +1031,10 @@ int vans_set_adjoint_launch(vans_t h, const vans_launch *cfg) {
         if (cfg->warps < 1 || cfg->rows < 1 || cfg->warps * cfg->rows > 8) return VANS_ERR_ARG;
         if (!(cfg->cpt == 1 || (cfg->cpt == 2 && h->q == 9))) return VANS_ERR_ARG;
     } else if (cfg->kind == 1) {
-        // pipeline: 2 or 4 compute warps, 2..8 stages; shapes with an instance
+        // pipeline: 2 or 4 compute warps (D3Q19 2..7), 2..8 stages; shapes with an instance
         const int nt = 32 * cfg->warps;
         const bool ok = h->q == 9 ? ((nt == 64 && cfg->cpt == 1) || (nt == 128 && cfg->cpt <= 2))
-                                  : (nt == 128 && cfg->cpt == 1);
+                                  : (nt >= 64 && nt <= 224 && cfg->cpt == 1);
         if (!ok || cfg->rows < 2 || cfg->rows > 8) return VANS_ERR_ARG;
     } else {
         return VANS_ERR_ARG;
