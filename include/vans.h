@@ -113,8 +113,11 @@ typedef struct {
  * kind 8: every step of a vans_step call in ONE launch of one thread-block
  *         cluster (up to `rows` CTAs, 2..16; `warps` 8 or 16 per CTA; cpt 1)
  *         that keeps the whole state in its distributed shared memory for the
- *         run, one cluster barrier per step: for domains of a few hundred KB,
- *         whose single-step launches cost more than their work.  Accepted
+ *         run: for domains of a few hundred KB, whose single-step launches
+ *         cost more than their work.  D2Q9 domains with two adjacent cells per
+ *         thread (other roundings than the single-step kinds; the forward
+ *         steps of vans_step_single and vans_adjoint_segment keep one cell
+ *         per thread and the single-step roundings).  Accepted
  *         only if the cluster holds the domain (D2Q9: at most 2 cells per
  *         thread, D3Q19: 1; two copies of each CTA's rows within 227 KB):
  *         VANS_ERR_UNSUPPORTED otherwise.  Plates on nodes included.
@@ -189,7 +192,8 @@ int vans_set_eps_async(vans_t h, const float *eps_dev);
  * f_i(x, t) of the current state: a porosity that varies in time, the
  * direction the paper names for two-fluid models (its concluding section).
  * The stored deviations are re-expressed for the new eps in place.
- * Synchronises once to check the range.  VANS_ERR_STATE before vans_set_eps. */
+ * Waits once for the range check, whose result comes through a pinned word that
+ * the handle allocates at the first call.  VANS_ERR_STATE before vans_set_eps. */
 int vans_update_eps(vans_t h, const float *eps_dev);
 
 /* ----------------------------------------------------------- time step -- */
@@ -206,7 +210,8 @@ int vans_step(vans_t h, int nsteps);
  * Errors as vans_step. */
 int vans_step_single(vans_t h, int nsteps);
 
-/* nsteps steps that watch themselves (no extra pass over the populations):
+/* nsteps steps that watch themselves (the step itself emits; with kind 9 and
+ * every > 1 one pass over the populations per emission, between launches):
  * the last step of every block of `every` steps (every >= 1; also the last of
  * the call) writes rho (dense N floats) and u (dense D*N floats) of the state
  * it reads -- the moments of Eqs. 0moment and 1moment, as vans_moments gives --

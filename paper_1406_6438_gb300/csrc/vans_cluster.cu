@@ -17,6 +17,12 @@
 // come after every read of step t.  The band is loaded from the state buffer
 // `fin` at the start and written back to `fout` at the end (columns -1 .. nx
 // of every row and direction, the library's padded layout).
+//
+// D2Q9 domains that fit take a second form, k_step_cluster_pair: two adjacent cells
+// per thread in packed arithmetic, the edge rows pushed to the neighbour instead of
+// pulled, no cluster barrier (0.547 us per step instead of 1.01 on the 128x64 channel).
+// The form above stays for D3Q19, for shapes that do not fit, and for the forward
+// steps of a reverse pass, which round as the single-step kernels do.
 #include <cooperative_groups.h>
 
 #include <type_traits>
