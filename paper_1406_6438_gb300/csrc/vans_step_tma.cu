@@ -25,10 +25,10 @@
 //      specialised as 4/5; 6 strided cells, 7 adjacent cells.  D3Q19 domains
 //      whose rows are not 256 cells are bound by too few warps for the
 //      arithmetic (12 per SM of kind 7 with 2 cells per thread, 127 registers)
-//      and by idle lanes: kind 6 takes one cell per thread (76 registers, 20
-//      warps) in tiles of 64 to 256 cells, rows of one tile without the staged
+//      and by idle lanes: kind 6 takes one cell per thread (64 registers, 24
+//      warps; 160 cells: 76 and 20) in tiles of 64 to 256 cells, rows of one tile without the staged
 //      halo columns: 150 x 110 x 90 58 -> 45 us (floor 34), 250^3 459 -> 392
-//      (360), 90^3 43 -> 27, 96 x 64 x 48 14.9 -> 11.6; 256^3 stays with kind 7
+//      (360), 90^3 43 -> 25.5, 96 x 64 x 48 14.9 -> 10.9; 256^3 stays with kind 7
 //      (397 against 414).
 //
 // (Kinds 1 -- a pipeline over contiguous runs of tiles with the porosity rows
@@ -677,8 +677,18 @@ __device__ __forceinline__ void ilv_run(Cur cur, const int *status, int ntiles, 
     }
 }
 
+// Blocks per SM to compile for (0: the compiler chooses; a 1 is another choice, 256^3
+// 428 us instead of 411): D3Q19 with one cell per thread fits in 64 registers, so as
+// many blocks as those allow (128^3 63.6 -> 61.1 us, 90^3 26.8 -> 25.5, 96 x 64 x 48
+// 11.3 -> 10.9, 221 x 150 x 150 131.8 -> 130.6), but for 160 cells, where a fifth block
+// costs more than it hides (150 x 110 x 90 44.8 -> 46.3).
+template <int Q, int NT, bool VEC, bool PL>
+__host__ __device__ constexpr int ilv_blocks() {
+    return Q == 19 && !VEC && !PL && NT != 160 ? 65536 / (NT + 32) / 64 : 0;
+}
+
 template <int Q, int NT, int CPT, bool VEC, bool PL = false, bool WRAP = false>
-__global__ void __launch_bounds__(NT + 32) k_step_tma_ilv(const VDom d, const float *__restrict__ fin,
+__global__ void __launch_bounds__(NT + 32, ilv_blocks<Q, NT, VEC, PL>()) k_step_tma_ilv(const VDom d, const float *__restrict__ fin,
                                                            float *__restrict__ fout, int ntx,
                                                            int ntiles, int stages) {
     extern __shared__ __align__(128) unsigned char smem[];
