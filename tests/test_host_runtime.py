@@ -1,0 +1,76 @@
+"""The host runtime on a CUDA runtime that runs nothing (host_runtime.cpp): which launches
+a call issues, and what it leaves behind when one of them fails."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import pytest
+
+from paper_1406_6438_gb300 import build as B
+from paper_1406_6438_gb300._binding import Params, _CLaunch
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ERR_ARG, ERR_CUDA, FAKE = -1, -2, ctypes.c_void_p(1 << 20)      # FAKE: never read or written
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("host") / "host_runtime.so")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(B._nvcc()))), "include")
+    subprocess.run([shutil.which("g++"), "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", B.INCLUDE,
+                    "-I", B.CSRC, "-isystem", cuda, "-include", "cstring", "-include", "cstdlib", "-x", "c++",
+                    os.path.join(B.CSRC, "vans_api.cu"), os.path.join(HERE, "host_runtime.cpp"), "-o", so], check=True)
+    so = ctypes.CDLL(so)
+    so.fake_log.restype = ctypes.c_char_p
+    so.vans_workspace_bytes.restype = so.vans_batch_workspace_bytes.restype = ctypes.c_size_t
+    return so
+
+
+class Handle:
+    """A handle with its porosity set; log() is what has been launched since the last."""
+
+    def __init__(self, lib, launch=None, **kw):
+        self.lib, self.h = lib, ctypes.c_void_p()
+        lib.fake_reset()
+        p = Params(**dict(dict(q=9, nx=600, ny=400, tau=0.7), **kw)).c()
+        n = lib.vans_workspace_bytes(ctypes.byref(p))
+        assert lib.vans_create(ctypes.byref(p), FAKE, ctypes.c_size_t(n), None, ctypes.byref(self.h)) == 0
+        assert self("set_eps", FAKE) == 0
+        if launch:
+            assert self("set_launch", ctypes.byref(_CLaunch(*launch))) == 0
+        self.log()
+
+    def __call__(self, name, *a):
+        return getattr(self.lib, "vans_" + name)(self.h, *a)
+
+    def log(self):
+        lines = self.lib.fake_log().decode().split("\n")[:-1]
+        self.lib.fake_reset()
+        return lines
+
+    def steps(self):
+        return sum(int(s.split()[1]) for s in self.log() if s.split()[0] in ("step", "multi", "cluster", "monitor"))
+
+
+KINDS = [(4, 4, 1, 0, 0), (2, 4, 4, 9, 0), (2, 4, 3, 9, 0), (2, 4, 2, 9, 0)]
+
+
+@pytest.mark.parametrize("launch", KINDS)
+@pytest.mark.parametrize("what", ["capture", "instantiate"])
+@pytest.mark.parametrize("nth", [1, 2])
+def test_a_failed_capture_runs_no_step(lib, launch, what, nth):
+    """Graphs of several sizes serve a run: where one of them cannot be made, none of the
+    run's steps has been issued, and the run can be asked for again."""
+    for warm in (0, 1):
+        h = Handle(lib, launch)
+        h("step", warm)
+        h.log()
+        for call in (("step", 63 * launch[2]), ("step_monitored", 190, 63, FAKE, FAKE, FAKE)):
+            h.log()
+            lib.fake_fail(what.encode(), nth)
+            assert h(*call) == ERR_CUDA
+            assert h.steps() == 0
+            assert h("step", 0) == 0 and h.steps() == 0
+        assert h("step", 63 * launch[2]) == 0
+        assert h.steps() == 63 * launch[2]
