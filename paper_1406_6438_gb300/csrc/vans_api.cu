@@ -361,7 +361,7 @@ void split_steps(vans_t h, int nsteps, Part p[2]) {
     p[0] = Part{nsteps, 1, h->gexec};
     p[1] = Part{0, 1, nullptr};
     if (h->L.kind != 9 || h->slab || nsteps < 2) return;
-    const int most = h->L.rows, launches = (nsteps + most - 1) / most;
+    const int most = h->L.rows, launches = 1 + (nsteps - 1) / most;
     const int few = nsteps / launches, longer = nsteps - few * launches;
     p[0] = Part{longer, few + 1, few + 1 == most ? h->gmulti : nullptr};
     p[1] = Part{launches - longer, few, few == most ? h->gmulti : nullptr};

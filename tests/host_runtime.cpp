@@ -13,9 +13,17 @@ std::vector<std::string> g_log, *g_into = &g_log;   // the capture's list while 
 std::map<std::string, int> g_fail;                  // calls until this one fails (1: the next)
 std::vector<std::vector<std::string>> g_graphs;
 std::string g_text;
-bool g_user_capture = false;
+bool g_user_capture = false, g_quiet = false;       // quiet: steps are counted, not logged
+long long g_steps = 0;
+std::vector<long long> g_graph_steps;
 
-void put(const std::string &s) { g_into->push_back(s); }
+void put(const std::string &s) {
+    const size_t at = s.find_first_of("0123456789");
+    const bool steps = s.compare(0, 4, "step") == 0 || s.compare(0, 5, "multi") == 0 ||
+                       s.compare(0, 7, "cluster") == 0 || s.compare(0, 7, "monitor") == 0;
+    if (steps) (g_into == &g_log ? g_steps : g_graph_steps.back()) += atoi(s.c_str() + at);
+    if (!g_quiet || g_into != &g_log) g_into->push_back(s);
+}
 cudaError_t call(const char *name) {
     auto f = g_fail.find(name);
     if (f != g_fail.end() && f->second > 0 && --f->second == 0) return cudaErrorUnknown;
@@ -35,8 +43,11 @@ void fake_reset() {
     g_log.clear();
     g_fail.clear();
     g_into = &g_log;
-    g_user_capture = false;
+    g_user_capture = g_quiet = false;
+    g_steps = 0;
 }
+void fake_quiet() { g_quiet = true; }
+long long fake_steps() { return g_steps; }
 void fake_fail(const char *name, int after) { g_fail[name] = after; }
 void fake_user_capture(int on) { g_user_capture = on != 0; }
 const char *fake_log() {
@@ -69,6 +80,7 @@ cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *s) {
 cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) {
     if (call("capture") != cudaSuccess) return cudaErrorUnknown;
     g_graphs.emplace_back();
+    g_graph_steps.push_back(0);
     g_into = &g_graphs.back();
     return cudaSuccess;
 }
@@ -84,7 +96,9 @@ cudaError_t cudaGraphInstantiate(cudaGraphExec_t *e, cudaGraph_t g, unsigned lon
 cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
 cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
 cudaError_t cudaGraphLaunch(cudaGraphExec_t e, cudaStream_t) {
-    for (const auto &s : g_graphs[(size_t)e - 1]) g_log.push_back(s);
+    g_steps += g_graph_steps[(size_t)e - 1];
+    if (!g_quiet)
+        for (const auto &s : g_graphs[(size_t)e - 1]) g_log.push_back(s);
     return call("graph");
 }
 cudaError_t cudaMemsetAsync(void *, int, size_t, cudaStream_t) { return logged("memset"); }

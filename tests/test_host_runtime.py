@@ -22,7 +22,7 @@ def lib(tmp_path_factory):
                     "-I", B.CSRC, "-isystem", cuda, "-include", "cstring", "-include", "cstdlib", "-x", "c++",
                     os.path.join(B.CSRC, "vans_api.cu"), os.path.join(HERE, "host_runtime.cpp"), "-o", so], check=True)
     so = ctypes.CDLL(so)
-    so.fake_log.restype = ctypes.c_char_p
+    so.fake_log.restype, so.fake_steps.restype = ctypes.c_char_p, ctypes.c_longlong
     so.vans_workspace_bytes.restype = so.vans_batch_workspace_bytes.restype = ctypes.c_size_t
     return so
 
@@ -50,7 +50,9 @@ class Handle:
         return lines
 
     def steps(self):
-        return sum(int(s.split()[1]) for s in self.log() if s.split()[0] in ("step", "multi", "cluster", "monitor"))
+        n = self.lib.fake_steps()
+        self.lib.fake_reset()
+        return n
 
 
 KINDS = [(4, 4, 1, 0, 0), (2, 4, 4, 9, 0), (2, 4, 3, 9, 0), (2, 4, 2, 9, 0)]
@@ -74,3 +76,12 @@ def test_a_failed_capture_runs_no_step(lib, launch, what, nth):
             assert h("step", 0) == 0 and h.steps() == 0
         assert h("step", 63 * launch[2]) == 0
         assert h.steps() == 63 * launch[2]
+
+
+@pytest.mark.parametrize("launch", KINDS)
+@pytest.mark.parametrize("n", [0, 1, 2, 3, 5, 9, 131, 2**31 - 1])
+def test_a_run_takes_the_steps_it_was_asked_for(lib, launch, n):
+    h = Handle(lib, launch)
+    lib.fake_quiet()
+    assert h("step", n) == 0
+    assert h.steps() == n
