@@ -193,7 +193,8 @@ int vans_set_eps_async(vans_t h, const float *eps_dev);
  * direction the paper names for two-fluid models (its concluding section).
  * The stored deviations are re-expressed for the new eps in place.
  * Waits once for the range check, whose result comes through a pinned word that
- * the handle allocates at the first call.  VANS_ERR_STATE before vans_set_eps. */
+ * the handle allocates at the first call: VANS_ERR_CUDA, and nothing enqueued, while
+ * the stream is captured.  VANS_ERR_STATE before vans_set_eps. */
 int vans_update_eps(vans_t h, const float *eps_dev);
 
 /* ----------------------------------------------------------- time step -- */

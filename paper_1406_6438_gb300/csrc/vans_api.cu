@@ -758,6 +758,10 @@ int vans_update_eps(vans_t h, const float *eps_dev) {
     if (!h || h->batched || !eps_dev) return VANS_ERR_ARG;
     if (!h->eps_set) return VANS_ERR_STATE;
     if (h->slab) return VANS_ERR_UNSUPPORTED;
+    // a captured stream cannot be waited for: refused before anything of it is recorded
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone)
+        return VANS_ERR_CUDA;
     if (const int rc = host_flag(h)) return rc;
     if (cudaMemsetAsync(h->flag, 0, sizeof(int), h->stream) != cudaSuccess) return VANS_ERR_CUDA;
     h->launches += 3;

@@ -85,3 +85,17 @@ def test_a_run_takes_the_steps_it_was_asked_for(lib, launch, n):
     lib.fake_quiet()
     assert h("step", n) == 0
     assert h.steps() == n
+
+
+@pytest.mark.parametrize("warm", [False, True])
+def test_update_eps_is_refused_under_capture(lib, warm):
+    """It has to wait for its range check.  The refusal leaves nothing in the capture: the
+    caller's graph would update the state of a call that failed."""
+    h = Handle(lib)
+    if warm:
+        assert h("update_eps", FAKE) == 0
+        assert h.log()[-2:] == ["rebase", "pad"]
+    lib.fake_user_capture(1)
+    assert h("update_eps", FAKE) == ERR_CUDA
+    assert h.log() == []
+    assert h("update_eps", FAKE) == 0
