@@ -227,9 +227,9 @@ template <int Q, int NT, int CPT, typename T>
 static cudaError_t launch_adj_tma_t(const VDom &d, const float *state, const float *lam_in,
                                     float *lam_out, float *grad, int stages, cudaStream_t s) {
     constexpr int TW = NT * CPT;
-    constexpr int NS = 2 * Q + EpsRows<Q>::N;
-    const size_t smem = kBarBytes + (size_t)stages * NS * (TW + 2 * kLead) * sizeof(float);
-    if (stages < 2 || stages > kBarBytes / 16 || smem > 227 * 1024) return cudaErrorInvalidValue;
+    static_assert(2 * Q + EpsRows<Q>::N == (Q == 9 ? 21 : 47), "rows of a stage (adjoint_smem)");
+    const size_t smem = adjoint_smem(Q, Launch{CPT, NT / 32, stages, 1});
+    if (stages < 2 || stages > kBarBytes / 16 || smem > kSmemMax) return cudaErrorInvalidValue;
     auto kern = k_adjoint_tma<Q, NT, CPT, T>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

@@ -1090,6 +1090,8 @@ int vans_set_adjoint_launch(vans_t h, const vans_launch *cfg) {
         const bool ok = h->q == 9 ? ((nt == 64 && cfg->cpt == 1) || (nt == 128 && cfg->cpt <= 2))
                                   : (nt >= 64 && nt <= 224 && cfg->cpt == 1);
         if (!ok || cfg->rows < 2 || cfg->rows > 8) return VANS_ERR_ARG;
+        if (vans::adjoint_smem(h->q, Launch{cfg->cpt, cfg->warps, cfg->rows, 1}) > (size_t)vans::kSmemMax)
+            return VANS_ERR_ARG;
     } else {
         return VANS_ERR_ARG;
     }

@@ -62,7 +62,19 @@ struct Launch {
     int ctas;
 };
 
+// Shared memory per CTA, the room for up to 16 mbarriers in front of a pipeline's
+// stages, and the columns staged on either side of a row segment: the +-1 neighbours of
+// its cells (halo columns included), from and to whole 32-byte sectors.
+constexpr int kSmemMax = 227 * 1024;
+constexpr int kBarBytes = 128;
+constexpr int kLead = 8;
+
 // ------------------------------------------------------- host helpers ----
+// Shared memory of the pipelined reverse step: L.rows stages of the populations, lambdas
+// and porosity rows (2 x 9 + 3, 2 x 19 + 9) of 32 * warps * cpt cells.
+inline size_t adjoint_smem(int q, const Launch &L) {
+    return kBarBytes + (size_t)L.rows * (q == 9 ? 21 : 47) * (32 * L.warps * L.cpt + 2 * kLead) * sizeof(float);
+}
 // Floats from a row's start to its column 0 for lattice q (VDom::off).
 inline int col0_for(int q) { return q == 19 ? 32 : 8; }
 // Floats per padded row for a row of nx cells: column 0 at col0_for(q),

@@ -34,13 +34,9 @@ __device__ __forceinline__ void row_nbs(const VDom &d, int row, int &y, int &z, 
     }
 }
 
-constexpr int kBarBytes = 128;   // room for up to 16 mbarriers in front of the stages
-
 // A staged row segment of the tile at column xs holds columns xs - kLead ..
-// xs + TW + kLead - 1: the +-1 neighbours of the tile's cells (halo columns
-// included), from and to whole 32-byte sectors (column 0 starts a sector, so
-// column xs - kLead starts one too); a stage slot is TW + 2 kLead floats.
-constexpr int kLead = 8;
+// xs + TW + kLead - 1 (column 0 starts a sector, so column xs - kLead starts one
+// too); a stage slot is TW + 2 kLead floats.
 
 // bytes of the copy of one staged row segment with nval cells
 __host__ __device__ constexpr uint32_t seg_bytes(int nval) {

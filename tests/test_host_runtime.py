@@ -99,3 +99,13 @@ def test_update_eps_is_refused_under_capture(lib, warm):
     assert h("update_eps", FAKE) == ERR_CUDA
     assert h.log() == []
     assert h("update_eps", FAKE) == 0
+
+
+def test_a_reverse_shape_that_does_not_fit_is_refused(lib):
+    """Stages that exceed 227 KB were accepted here and failed at every launch."""
+    h = Handle(lib, q=19, nx=40, ny=5, nz=3)
+    most = {2: 8, 3: 8, 4: 8, 5: 7, 6: 5, 7: 5}
+    for warps in range(2, 8):
+        for stages in range(2, 9):
+            rc = h("set_adjoint_launch", ctypes.byref(_CLaunch(1, warps, stages, 1, 0)))
+            assert rc == (0 if stages <= most[warps] else ERR_ARG), (warps, stages)
