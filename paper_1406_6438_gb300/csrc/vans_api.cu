@@ -925,10 +925,12 @@ int vans_autotune(vans_t h, vans_launch *chosen) {
         if (L.kind == 9 && !vans::multi_fits(h->q, h->dom)) continue;
         // D3Q19, one cell per thread: of the tile widths only the one that takes a row
         // in the fewest tiles with the fewest idle lanes (beside 128 and 256 cells with
-        // 3 stages).  150 x 110 x 90: 160 cells 45.0 us, 192 51, 224 62, 96 (two tiles) 61
+        // 3 stages).  150 x 110 x 90: 160 cells 45.0 us, 192 51, 224 62, 96 (two tiles) 61.
+        // Up to 32 cells: the 64-cell tile, though kind 0 is faster (32 x 128 x 128: 37.6
+        // against 32.7; the 128-cell tile 59.0)
         const int tiles = (h->dom.nx + 255) / 256, cells = (h->dom.nx + tiles - 1) / tiles;
         if (h->q == 19 && L.kind == 6 && (L.rows == 2 || L.warps % 4 != 0) &&
-            (cells + 31) / 32 != L.warps)
+            std::max(2, (cells + 31) / 32) != L.warps)
             continue;
         // all scored as the time of `reps` steps
         float ms = 1e30f;

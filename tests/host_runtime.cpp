@@ -112,7 +112,7 @@ cudaError_t cudaMemcpyAsync(void *to, const void *, size_t n, cudaMemcpyKind kin
 namespace vans {
 
 cudaError_t launch_step(int, const VDom &, const float *, float *, Launch L, cudaStream_t) {
-    return logged("step 1 kind " + num(L.kind));
+    return logged("step 1 kind " + num(L.kind) + " warps " + num(L.warps) + " rows " + num(L.rows));
 }
 cudaError_t launch_multi(const VDom &, const float *, float *, int steps, int, cudaStream_t) {
     return logged("multi " + num(steps));

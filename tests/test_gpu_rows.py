@@ -55,3 +55,13 @@ def test_halo_copies_serve_the_other_kinds(nx):
         s.close()
     for f in out[1:]:
         assert torch.equal(f, out[0])
+
+
+@pytest.mark.parametrize("nx", [1, 24, 31, 32])
+def test_the_narrowest_tile_takes_short_rows(nx):
+    """Rows of at most half the 64-cell tile, which autotune offers them."""
+    p, eps, f0 = _case(nx, 6, seed=nx)
+    rho_o, u_o, f_o = oracle_run(p, eps, 5, f0)
+    for stages in (2, 3):
+        rho, u, f = gpu_run(p, eps, 5, f0, launch=Launch(1, 2, stages, 6))
+        assert np.abs(f - f_o).max() <= 2e-7 and rel_u(u, u_o) <= 1e-5

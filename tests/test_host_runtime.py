@@ -109,3 +109,13 @@ def test_a_reverse_shape_that_does_not_fit_is_refused(lib):
         for stages in range(2, 9):
             rc = h("set_adjoint_launch", ctypes.byref(_CLaunch(1, warps, stages, 1, 0)))
             assert rc == (0 if stages <= most[warps] else ERR_ARG), (warps, stages)
+
+
+@pytest.mark.parametrize("nx,warps", [(1, 2), (24, 2), (32, 2), (64, 2), (65, 3), (150, 5), (256, 8), (300, 5)])
+def test_autotune_tries_the_tile_that_fits_the_rows(lib, nx, warps):
+    """Of the D3Q19 tiles with one cell per thread and 2 stages: the narrowest of 64 to 256
+    cells that takes a row in as few tiles as there can be."""
+    h = Handle(lib, q=19, nx=nx, ny=40, nz=30)
+    assert h("autotune", None) == 0
+    tried = {tuple(s.split()[2:]) for s in h.log() if s.startswith("step 1 kind 6")}
+    assert [t[3] for t in tried if t[5] == "2"] == [str(warps)], tried
