@@ -505,7 +505,9 @@ __global__ void __launch_bounds__(256) k_step_adjoint(const VDom d, const float 
         adj_row<Q, CPT, false, T>(d, st, lin, lout, grad, y, z, x0, lane);
 }
 
-// A sum held as two floats, head and tail (Knuth's two-sum; 48 bits).
+// A sum held as two floats, head and tail (Knuth's two-sum; 48 bits).  The product of
+// add_scaled is rounded by itself: contracted into the two-sum's additions, its rounding
+// would be in the tail twice (24 bits of a scaled sum).
 struct TwoFloat {
     float h = 0.f, l = 0.f;
     __device__ __forceinline__ void add(float a) {
@@ -515,7 +517,7 @@ struct TwoFloat {
     }
     // w times the sum t, the rounding of w * t.h included
     __device__ __forceinline__ void add_scaled(float w, const TwoFloat &t) {
-        const float p = w * t.h;
+        const float p = __fmul_rn(w, t.h);
         add(p);
         l += fmaf(w, t.h, -p) + w * t.l;
     }

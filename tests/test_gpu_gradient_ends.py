@@ -3,6 +3,7 @@ grad-eps stencil, against float64 sums of the same numbers."""
 import numpy as np
 import pytest
 
+import oracle as O
 from paper_1406_6438_gb300 import workloads as W
 from tests._gpu import solver, torch_cuda
 
@@ -77,3 +78,65 @@ def test_gradient_stencil(q, shape, walls):
         for field, where in ((src, ~past(-1)), (G, past(1))):
             v += np.where(where, 3 * w * sum(e[c] * field[1 + c] for c in range(D)), 0.0)
     assert np.all(np.abs(out - v) <= 2.0 ** -23 * np.abs(v) + 2.0 ** -42 * 1e4 * 36)
+
+
+def _stencil64(q, shape, walls, lam, G):
+    """G_eps + sum w lambda + the transposed stencil in 64 bits; lam[i]: plane i of the
+    lambda state, G: the accumulators' sums."""
+    e, w, opp = O.lattice(q)[:3]
+    w = np.asarray(w, dtype=np.float32).astype(np.float64)
+    nz, ny, nx = shape
+    z, y, x = np.meshgrid(*(np.arange(n) for n in shape), indexing="ij")
+    v = G[0].astype(np.float64)
+    for i, ei in enumerate(np.asarray(e)):
+        ei = list(ei) + [0] * (3 - len(ei))
+
+        def past(sign):
+            yy, zz = y + sign * ei[1], z + sign * ei[2]
+            return ((walls & 2 != 0) & ((yy < 0) | (yy >= ny))) | ((walls & 4 != 0) & ((zz < 0) | (zz >= nz)))
+
+        def src(f):
+            return f[..., (z - ei[2]) % nz, (y - ei[1]) % ny, (x - ei[0]) % nx]
+        v += w[i] * np.where(past(-1), lam[opp[i]], src(lam[i]))
+        for field, where in ((src(G), ~past(-1)), (G, past(1))):
+            v += np.where(where, 3 * w[i] * sum(ei[c] * field[1 + c] for c in range(len(G) - 1) if ei[c]), 0.0)
+    return v
+
+
+def _finalize(q, shape, walls, lam, acc, bits=32):
+    torch = torch_cuda()
+    p, eps, _ = _case(q, shape, walls, seed=2)
+    s = solver(p, eps)
+    s.set_adjoint_precision(bits)
+    rows, off = shape[0] * shape[1], 8 if q == 9 else 32
+    pitch = s.state_floats // (q * rows) // 32 * 32           # (the state's end is padded too)
+    state = s.new_state()
+    lam = np.concatenate([lam[..., -1:], lam, lam[..., :1]], axis=-1).reshape(q, rows, -1)   # halo columns
+    state[:q * rows * pitch].view(q, rows, pitch)[:, :, off - 1:off + shape[2] + 1] = torch.from_numpy(lam).cuda()
+    return s.grad_finalize(state, torch.from_numpy(acc.ravel()).cuda()).cpu().numpy().reshape(shape)
+
+
+def _cancelling(q, shape, rng, noise):
+    """lambda of 1e4 whose weighted sum cancels to about `noise`."""
+    lam = np.empty((q,) + shape)
+    w0 = float(np.float32(4 / 9 if q == 9 else 1 / 3))
+    lam[0] = 1e4
+    lam[1:] = -1e4 * w0 / (1 - w0)
+    return (lam + noise * rng.standard_normal((q,) + shape)).astype(np.float32)
+
+
+@pytest.mark.parametrize("walls", [0, 2, 6])
+@pytest.mark.parametrize("q,shape", SHAPES)
+def test_lambda_and_stencil_cancel(q, shape, walls):
+    """lambda of 1e4 whose weighted sums cancel, against a stencil that cancels too: half
+    an ulp of the result, and 2^-42 of the terms for the two-float sums of 55."""
+    if q == 9 and walls == 6:
+        pytest.skip("no z walls in two dimensions")
+    rng, D = np.random.default_rng(6), 2 if q == 9 else 3
+    lam = _cancelling(q, shape, rng, 1.0)
+    head = (1e4 + rng.standard_normal((1 + D,) + shape)).astype(np.float32)
+    head[0] = rng.standard_normal(shape)
+    tail = (1e-4 * rng.standard_normal((1 + D,) + shape)).astype(np.float32)
+    out = _finalize(q, shape, walls, lam, np.stack([head, tail]))
+    v = _stencil64(q, shape, walls, lam.astype(np.float64), head.astype(np.float64) + tail)
+    assert np.all(np.abs(out - v) <= 2.0 ** -24 * np.abs(v) + 2.0 ** -42 * 1e4 * 55)
