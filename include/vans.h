@@ -300,8 +300,9 @@ int vans_adjoint_segment(vans_t h, const float *ckpt, float *seg, int len, float
  * of shared memory hold); ctas must be 0.  VANS_ERR_ARG otherwise. */
 int vans_set_adjoint_launch(vans_t h, const vans_launch *cfg);
 
-/* Arithmetic of the per-cell reverse step: 32 (FP32, the default) or 64 (FP64;
- * loads, stores and the compensated accumulation stay FP32).  The eps gradient
+/* Arithmetic of the per-cell reverse step and of the sums of vans_grad_finalize: 32
+ * (FP32, those sums in two floats; the default) or 64 (FP64; loads, stores and the
+ * compensated accumulation stay FP32).  The eps gradient
  * is a small residual of large grad-eps sensitivities, so FP32 per-cell
  * rounding limits its relative accuracy on long rollouts.  VANS_ERR_ARG for
  * other values. */

@@ -1117,7 +1117,7 @@ int vans_grad_finalize(vans_t h, const float *lam0, const float *grad_acc, float
     if (!h->eps_set) return VANS_ERR_STATE;
     ++h->launches;
     return cuda_status(
-        vans::launch_grad_finalize(h->q, h->dom, lam0, grad_acc, dJdeps_dev, h->stream));
+        vans::launch_grad_finalize(h->q, h->dom, lam0, grad_acc, dJdeps_dev, h->adj_fp64, h->stream));
 }
 
 int vans_check(vans_t h) {

@@ -527,9 +527,48 @@ struct TwoFloat {
 // grad-eps stencil applied to G_grad.  Runs once per reverse pass; the stencil's
 // terms cancel to a much smaller result, so it combines the compensated accumulators
 // (sum + compensation) and evaluates the stencil as two-float sums, one per weight
-// (axis and diagonal directions), scaled at the end.  In FP64 the kernel was bound by
-// that pipe, of 1/64 of the FP32 rate: 96 x 64 x 48 175 us, 512^2 59 us (now 38, 14).
+// (axis and diagonal directions), scaled at the end.  In FP64 the kernel is bound by
+// that pipe, of 1/64 of the FP32 rate: back to back 112 us at 96 x 64 x 48 and 54 at
+// 512^2, as two floats 29.4 and 12.7; the sums are in FP64 where the caller asked for that
+// arithmetic (vans_set_adjoint_precision).
+
+// the gradient of cell n = (x, y, z) with every sum in FP64
 template <int Q>
+__device__ double cell_gradient64(const VDom &d, const float *__restrict__ lam0,
+                                  const float *__restrict__ grad, long long n, int x, int y, int z) {
+    using L = Lat<Q>;
+    constexpr int D = L::D;
+    const long long nc = (1 + D) * d.cells;
+    auto G = [&](int comp, long long m) { return (double)grad[comp * d.cells + m] + (double)grad[nc + comp * d.cells + m]; };
+    Nb3 Y, Z;
+    nb_yz<Q>(d, y, z, Y, Z);
+    double v = G(0, n);
+#pragma unroll
+    for (int i = 0; i < Q; ++i)
+        v += (double)L::w(i) * (double)lam0[pull_index<Q>(d, i, x, y, z, Y, Z)];
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+        const int e[3] = {L::ex(i), L::ey(i), L::ez(i)};
+        auto term = [&](long long m) {                      // e_i . G_grad(m)
+            double s = 0.0;
+#pragma unroll
+            for (int c = 0; c < D; ++c)
+                if (e[c]) s += e[c] * G(1 + c, m);
+            v += 3.0 * (double)L::w(i) * s;
+        };
+        // cell x - e_i, whose stencil reads eps(x) through direction i
+        if (!(Y.wall[1 - e[1]] || Z.wall[1 - e[2]])) {
+            int xs = x - e[0];
+            xs = xs < 0 ? xs + d.nx : (xs >= d.nx ? xs - d.nx : xs);
+            term(((long long)Z.r[1 - e[2]] * d.ny + Y.r[1 - e[1]]) * d.nx + xs);
+        }
+        // x itself, whose neighbour x + e_i lies past a wall
+        if (Y.wall[1 + e[1]] || Z.wall[1 + e[2]]) term(n);
+    }
+    return v;
+}
+
+template <int Q, bool FP64>
 __global__ void __launch_bounds__(256)
     k_grad_finalize(const VDom d, const float *__restrict__ lam0, const float *__restrict__ grad,
                     float *__restrict__ out) {
@@ -540,6 +579,10 @@ __global__ void __launch_bounds__(256)
          n += (long long)gridDim.x * blockDim.x) {
         int x, y, z;
         cell_xyz(d, n, x, y, z);
+        if (FP64) {
+            out[n] = (float)cell_gradient64<Q>(d, lam0, grad, n, x, y, z);
+            continue;
+        }
         Nb3 Y, Z;
         nb_yz<Q>(d, y, z, Y, Z);
         TwoFloat sa, sd, la, ld, v;
@@ -787,10 +830,11 @@ cudaError_t launch_step_adjoint(int q, const VDom &d, const float *state, const 
 }
 
 cudaError_t launch_grad_finalize(int q, const VDom &d, const float *lam0, const float *grad,
-                                 float *dJ, cudaStream_t s) {
+                                 float *dJ, int fp64, cudaStream_t s) {
     const int g = grid_for(d.cells, 256);
-    VANS_DISPATCH_Q(q, (k_grad_finalize<9><<<g, 256, 0, s>>>(d, lam0, grad, dJ)),
-                    (k_grad_finalize<19><<<g, 256, 0, s>>>(d, lam0, grad, dJ)));
+    auto kern = q == 9 ? (fp64 ? k_grad_finalize<9, true> : k_grad_finalize<9, false>)
+                       : (fp64 ? k_grad_finalize<19, true> : k_grad_finalize<19, false>);
+    kern<<<g, 256, 0, s>>>(d, lam0, grad, dJ);
     return cudaGetLastError();
 }
 

@@ -153,7 +153,7 @@ cudaError_t launch_step_adjoint(int q, const VDom &d, const float *state, const 
                                 float *lam_out, float *grad, int fp64, Launch L,
                                 cudaStream_t stream);
 cudaError_t launch_grad_finalize(int q, const VDom &d, const float *lam0, const float *grad,
-                                 float *dJ, cudaStream_t stream);
+                                 float *dJ, int fp64, cudaStream_t stream);
 // kind 9 over a batch: CTA table {dom, first of four units, column blocks, strips}
 // built for launches of table_steps steps, whose blocks store multi_out_cols columns
 constexpr int kMultiWarps = 4;

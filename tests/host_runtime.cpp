@@ -140,7 +140,7 @@ cudaError_t launch_flux_seed(int, const VDom &, const float *, int, float *, flo
 cudaError_t launch_step_adjoint(int, const VDom &, const float *, const float *, float *, float *, int, Launch, cudaStream_t) {
     return logged("reverse 1");
 }
-cudaError_t launch_grad_finalize(int, const VDom &, const float *, const float *, float *, cudaStream_t) {
+cudaError_t launch_grad_finalize(int, const VDom &, const float *, const float *, float *, int, cudaStream_t) {
     return logged("stencil");
 }
 cudaError_t launch_ring_batched(const VDom *, const Tile *, int, int, Launch L, int *, cudaStream_t, unsigned long long *) {

@@ -140,3 +140,25 @@ def test_lambda_and_stencil_cancel(q, shape, walls):
     out = _finalize(q, shape, walls, lam, np.stack([head, tail]))
     v = _stencil64(q, shape, walls, lam.astype(np.float64), head.astype(np.float64) + tail)
     assert np.all(np.abs(out - v) <= 2.0 ** -24 * np.abs(v) + 2.0 ** -42 * 1e4 * 55)
+
+
+@pytest.mark.parametrize("walls", [0, 2, 6])
+@pytest.mark.parametrize("q,shape", [(9, (1, 40, 131)), (19, (9, 10, 67))])
+def test_64_bit_sums_where_they_are_asked_for(q, shape, walls):
+    """set_adjoint_precision(64): terms of at most 20 bits on a grid of 2^-6, so that every
+    product with a weight (24 bits) and every sum of 55 of them is exact in 64 bits,
+    cancelling to 1e-3: the result is the exact sum rounded once."""
+    if q == 9 and walls == 6:
+        pytest.skip("no z walls in two dimensions")
+    rng, D = np.random.default_rng(7), 2 if q == 9 else 3
+    grid = lambda a: (np.round(a * 64) / 64).astype(np.float32)  # noqa: E731
+    lam = grid(_cancelling(q, shape, rng, 0.1))
+    acc = np.zeros((2, 1 + D) + shape, dtype=np.float32)
+    acc[0, 1:] = grid(1e4 + rng.standard_normal((D,) + shape))
+    G = acc.astype(np.float64).sum(0)
+    G[0] = 0
+    acc[0, 0] = -grid(_stencil64(q, shape, walls, lam.astype(np.float64), G))
+    G[0] = acc[0, 0]
+    v = _stencil64(q, shape, walls, lam.astype(np.float64), G)
+    out = _finalize(q, shape, walls, lam, acc, bits=64)
+    assert np.all(np.abs(out - v) <= 2.0 ** -24 * np.abs(v))
