@@ -528,13 +528,13 @@ struct TwoFloat {
 // terms cancel to a much smaller result, so it combines the compensated accumulators
 // (sum + compensation) and evaluates the stencil as two-float sums, one per weight
 // (axis and diagonal directions), scaled at the end.  In FP64 the kernel is bound by
-// that pipe, of 1/64 of the FP32 rate: back to back 112 us at 96 x 64 x 48 and 54 at
-// 512^2, as two floats 29.4 and 12.7; the sums are in FP64 where the caller asked for that
+// that pipe, of 1/64 of the FP32 rate: back to back 108 us at 96 x 64 x 48 and 46 at
+// 512^2, as two floats 27.4 and 12.0; the sums are in FP64 where the caller asked for that
 // arithmetic (vans_set_adjoint_precision).
 
 // the gradient of cell n = (x, y, z) with every sum in FP64
 template <int Q>
-__device__ double cell_gradient64(const VDom &d, const float *__restrict__ lam0,
+__device__ __noinline__ double cell_gradient64(const VDom &d, const float *__restrict__ lam0,
                                   const float *__restrict__ grad, long long n, int x, int y, int z) {
     using L = Lat<Q>;
     constexpr int D = L::D;
@@ -623,7 +623,9 @@ __global__ void __launch_bounds__(256)
         sd3.add_scaled(3.f, sd);
         v.add_scaled(L::w(A), sa3);
         v.add_scaled(L::w(B), sd3);
-        out[n] = v.h + v.l;
+        // a sum that left the range of floats (its tail is NaN then): as FP64 sums it
+        const float sum = v.h + v.l;
+        out[n] = isfinite(sum) ? sum : (float)cell_gradient64<Q>(d, lam0, grad, n, x, y, z);
     }
 }
 

@@ -162,3 +162,27 @@ def test_64_bit_sums_where_they_are_asked_for(q, shape, walls):
     v = _stencil64(q, shape, walls, lam.astype(np.float64), G)
     out = _finalize(q, shape, walls, lam, acc, bits=64)
     assert np.all(np.abs(out - v) <= 2.0 ** -24 * np.abs(v))
+
+
+@pytest.mark.parametrize("bits", [32, 64])
+@pytest.mark.parametrize("q,shape", [(9, (1, 6, 9)), (19, (4, 5, 6))])
+def test_sums_that_leave_the_range_of_floats(q, shape, bits):
+    """An infinite or NaN accumulator or lambda gives what a sum in 64 bits gives, and terms
+    whose partial sums pass the largest float do not."""
+    D = 2 if q == 9 else 3
+    for kind in ("inf", "-inf", "nan", "large"):
+        lam = np.zeros((q,) + shape, dtype=np.float32)
+        acc = np.zeros((2, 1 + D) + shape, dtype=np.float32)
+        if kind == "large":
+            lam[:] = np.where(np.arange(q) % 2, 3e38, -3e38).reshape((q,) + (1,) * 3)
+            acc[0, 1:] = 3e38 * np.sign(np.arange(acc[0, 1:].size) % 3 - 1.0).reshape(acc[0, 1:].shape)
+        else:
+            acc[0, 0, 0, 2, 3] = acc[0, 1, 0, 4, 4] = float(kind)
+            lam[3, 0, 1, 1] = float(kind)
+        with np.errstate(invalid="ignore", over="ignore"):
+            G = acc.astype(np.float64).sum(0)
+            v = _stencil64(q, shape, 2, lam.astype(np.float64), G).astype(np.float32)
+        out = _finalize(q, shape, 2, lam, acc, bits)
+        assert np.array_equal(np.isnan(out), np.isnan(v)), kind
+        ok = ~np.isnan(v)
+        assert np.allclose(out[ok], v[ok], rtol=1e-5, atol=1e-30), kind
