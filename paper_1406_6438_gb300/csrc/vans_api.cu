@@ -174,6 +174,7 @@ struct vans_s {
     Launch Ls{4, 4, 1, 0};                      // single steps: L, or its stand-in if L is kind 9
     cudaGraphExec_t gexec[kGraphSizes] = {};   // 64, 32, ..., 2 single-step launches
     cudaGraphExec_t gmulti[kGraphSizes] = {};  // as many kind 9 launches of L.rows steps
+    int strips[vans::kMultiMax + 1] = {};       // of a kind 9 launch of 2..L.rows steps
     int *flag = nullptr;                        // device status words (workspace)
     int *flag_host = nullptr;                   // pinned copy of flag[0] (vans_update_eps)
     cudaEvent_t flag_read = nullptr;            // behind that copy
@@ -245,12 +246,21 @@ cudaError_t batched_multi(vans_t h, cudaStream_t s, int par, int steps) {
 // the single-step launch of a handle that nobody has tuned
 Launch single_default(int q) { return q == 9 ? Launch{4, 4, 1, 0} : Launch{2, 4, 1, 0}; }
 
+// the strips of the kind 9 launches of L
+int set_strips(vans_t h, const Launch &L) {
+    int n[vans::kMultiMax + 1] = {};
+    for (int k = 2; k <= L.rows; ++k)
+        if (vans::multi_strips(h->dom, k, L.ctas, &n[k]) != cudaSuccess) return VANS_ERR_CUDA;
+    std::copy(std::begin(n), std::end(n), h->strips);
+    return VANS_OK;
+}
+
 // one launch of `steps` steps (more than one: kind 9)
 cudaError_t one_launch(vans_t h, cudaStream_t s, int par, int steps) {
     ++h->launches;
     if (h->batched) return steps > 1 ? batched_multi(h, s, par, steps) : batched_step(h, s, par);
     if (steps > 1)
-        return vans::launch_multi(h->dom, h->st[par], h->st[par ^ 1], steps, h->L.ctas, s);
+        return vans::launch_multi(h->dom, h->st[par], h->st[par ^ 1], steps, h->strips[steps], s);
     return vans::launch_step(h->q, h->dom, h->st[par], h->st[par ^ 1], h->Ls, s);
 }
 
@@ -901,6 +911,7 @@ int vans_set_launch(vans_t h, const vans_launch *cfg) {
         VDom whole = h->dom;         // a slab steps by single launches until the next vans_set_eps
         whole.xwrap = 1;
         if (!vans::multi_fits(h->q, whole)) return VANS_ERR_UNSUPPORTED;
+        if (const int rc = set_strips(h, L)) return rc;
     }
     h->L = L;
     h->Ls = L.kind == 9 ? single_default(h->q) : L;
@@ -937,8 +948,10 @@ int vans_autotune(vans_t h, vans_launch *chosen) {
         if (L.kind == 9) {
             // several launches in a row, as a run issues them
             const int n = std::max(2, reps / L.rows);
+            int strips = 0;
+            if (vans::multi_strips(h->dom, L.rows, L.ctas, &strips) != cudaSuccess) continue;
             ms = time_launches(h, [&](cudaStream_t st) {
-                return vans::launch_multi(h->dom, in, outb, L.rows, L.ctas, st);
+                return vans::launch_multi(h->dom, in, outb, L.rows, strips, st);
             }, n) * reps / (float)(n * L.rows);
             h->launches += 4 * n;
             if (ms < best_ms) {
@@ -979,6 +992,8 @@ int vans_autotune(vans_t h, vans_launch *chosen) {
         }
     }
     if (cudaGetLastError() != cudaSuccess) return VANS_ERR_CUDA;
+    if (best.kind == 9)
+        if (const int rc = set_strips(h, best)) return rc;
     h->L = best;
     h->Ls = best.kind >= 8 ? single : best;
     drop_graph(h);

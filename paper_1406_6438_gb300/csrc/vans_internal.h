@@ -106,12 +106,14 @@ cudaError_t launch_step_tma(int q, const VDom &d, const float *fin, float *fout,
 cudaError_t launch_step_cluster(int q, const VDom &d, const float *fin, float *fout, int nsteps,
                                 Launch L, bool pairs, cudaStream_t stream);
 // kind 9 (D2Q9, x periodic within the domain, no plates on nodes): `steps`
-// (2..kMultiMax) steps in one launch, in strips for `ctas` CTAs per SM (0: chosen)
+// (2..kMultiMax) steps in one launch, every column block cut into `strips` strips of rows
 constexpr int kMultiMax = 4;
 // whether kind 9 takes the domain: D2Q9, no plates on nodes, not a slab, planes
 // of less than 4 GB
 bool multi_fits(int q, const VDom &d);
-cudaError_t launch_multi(const VDom &d, const float *fin, float *fout, int steps, int ctas,
+// strips for `ctas` CTAs per SM (0: as many as fit)
+cudaError_t multi_strips(const VDom &d, int steps, int ctas, int *strips);
+cudaError_t launch_multi(const VDom &d, const float *fin, float *fout, int steps, int strips,
                          cudaStream_t stream);
 // whether a cluster of at most cmax CTAs of `warps` warps holds the domain
 // (never plates on nodes)

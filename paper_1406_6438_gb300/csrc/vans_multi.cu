@@ -423,23 +423,27 @@ struct Prepared {
 };
 
 template <int T, bool WALLS>
-cudaError_t launch_multi_t(const VDom &d, const float *fin, float *fout, int ctas,
-                           cudaStream_t stream) {
-    auto kern = k_multi<T, WALLS>;
+Prepared &prepared() {
     static Prepared ready;
+    return ready;
+}
+
+// Strips per column block: the count with the smallest waves x turns (a strip
+// of n rows takes n + 2 (T-1) turns, and its start is worth one more), a wave
+// being as many warps as the chip holds, or ctas blocks per SM in one wave:
+// fewer and longer strips repeat fewer rows, which is the better choice where
+// short strips would be half repetition (1024^2, T = 4: 9.0 us per step with
+// 3 blocks per SM, 8.4 with 1).  The search takes up to ny turns of the host (three launches
+// of 96 x 20000: 95 us of it, now 6.5), so a handle makes it when its shape is set.
+template <int T, bool WALLS>
+cudaError_t strips_t(const VDom &d, int ctas, int *strips) {
     int sms = 0, occ = 0;
-    const size_t smem = (size_t)kMultiWarps * warp_smem<T>();
-    const cudaError_t e = ready.get(kern, smem, sms, occ);
+    const cudaError_t e =
+        prepared<T, WALLS>().get(k_multi<T, WALLS>, (size_t)kMultiWarps * warp_smem<T>(), sms, occ);
     if (e != cudaSuccess) return e;
     const int ncol = (d.nx + out_cols(T) - 1) / out_cols(T);
-    // Strips per column block: the count with the smallest waves x turns (a strip
-    // of n rows takes n + 2 (T-1) turns, and its start is worth one more), a wave
-    // being as many warps as the chip holds, or ctas blocks per SM in one wave:
-    // fewer and longer strips repeat fewer rows, which is the better choice where
-    // short strips would be half repetition (1024^2, T = 4: 9.0 us per step with
-    // 3 blocks per SM, 8.4 with 1)
     const long long resident = (long long)sms * (ctas > 0 && ctas < occ ? ctas : occ) * kMultiWarps;
-    int nstrip = 1;
+    *strips = 1;
     double best = 1e300;
     for (int s = 1; s <= d.ny; ++s) {
         const long long units = (long long)ncol * s;
@@ -447,21 +451,25 @@ cudaError_t launch_multi_t(const VDom &d, const float *fin, float *fout, int cta
         const double cost = (double)waves * ((d.ny + s - 1) / s + 2 * (T - 1) + 1);
         if (cost < best) {
             best = cost;
-            nstrip = s;
+            *strips = s;
         }
         if (units > (ctas > 0 ? 1 : 8) * resident) break;
     }
-    const long long grid = ((long long)ncol * nstrip + kMultiWarps - 1) / kMultiWarps;
-    if (grid > 0x7fffffffLL / kMultiWarps) return cudaErrorInvalidConfiguration;
-    kern<<<(unsigned)grid, 32 * kMultiWarps, smem, stream>>>(d, fin, fout, ncol, nstrip);
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
-template <int T>
-cudaError_t launch_steps(const VDom &d, const float *fin, float *fout, int ctas,
-                         cudaStream_t stream) {
-    return d.wall_y ? launch_multi_t<T, true>(d, fin, fout, ctas, stream)
-                    : launch_multi_t<T, false>(d, fin, fout, ctas, stream);
+template <int T, bool WALLS>
+cudaError_t launch_multi_t(const VDom &d, const float *fin, float *fout, int strips,
+                           cudaStream_t stream) {
+    int sms = 0, occ = 0;
+    const size_t smem = (size_t)kMultiWarps * warp_smem<T>();
+    const cudaError_t e = prepared<T, WALLS>().get(k_multi<T, WALLS>, smem, sms, occ);
+    if (e != cudaSuccess) return e;
+    const int ncol = (d.nx + out_cols(T) - 1) / out_cols(T);
+    const long long grid = ((long long)ncol * strips + kMultiWarps - 1) / kMultiWarps;
+    if (strips < 1 || strips > d.ny || grid > 0x7fffffffLL / kMultiWarps) return cudaErrorInvalidConfiguration;
+    k_multi<T, WALLS><<<(unsigned)grid, 32 * kMultiWarps, smem, stream>>>(d, fin, fout, ncol, strips);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -499,13 +507,25 @@ bool multi_fits(int q, const VDom &d) {
     return q == 9 && !d.nee && d.xwrap && d.plane < (1LL << 30);
 }
 
-cudaError_t launch_multi(const VDom &d, const float *fin, float *fout, int steps, int ctas,
+cudaError_t multi_strips(const VDom &d, int steps, int ctas, int *strips) {
+    switch (steps) {
+        case 2: return d.wall_y ? strips_t<2, true>(d, ctas, strips) : strips_t<2, false>(d, ctas, strips);
+        case 3: return d.wall_y ? strips_t<3, true>(d, ctas, strips) : strips_t<3, false>(d, ctas, strips);
+        case 4: return d.wall_y ? strips_t<4, true>(d, ctas, strips) : strips_t<4, false>(d, ctas, strips);
+    }
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_multi(const VDom &d, const float *fin, float *fout, int steps, int strips,
                          cudaStream_t stream) {
     if (!multi_fits(9, d)) return cudaErrorInvalidValue;
     switch (steps) {
-        case 2: return launch_steps<2>(d, fin, fout, ctas, stream);
-        case 3: return launch_steps<3>(d, fin, fout, ctas, stream);
-        case 4: return launch_steps<4>(d, fin, fout, ctas, stream);
+        case 2: return d.wall_y ? launch_multi_t<2, true>(d, fin, fout, strips, stream)
+                                : launch_multi_t<2, false>(d, fin, fout, strips, stream);
+        case 3: return d.wall_y ? launch_multi_t<3, true>(d, fin, fout, strips, stream)
+                                : launch_multi_t<3, false>(d, fin, fout, strips, stream);
+        case 4: return d.wall_y ? launch_multi_t<4, true>(d, fin, fout, strips, stream)
+                                : launch_multi_t<4, false>(d, fin, fout, strips, stream);
     }
     return cudaErrorInvalidValue;
 }

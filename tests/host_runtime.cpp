@@ -114,8 +114,12 @@ namespace vans {
 cudaError_t launch_step(int, const VDom &, const float *, float *, Launch L, cudaStream_t) {
     return logged("step 1 kind " + num(L.kind) + " warps " + num(L.warps) + " rows " + num(L.rows));
 }
-cudaError_t launch_multi(const VDom &, const float *, float *, int steps, int, cudaStream_t) {
-    return logged("multi " + num(steps));
+cudaError_t launch_multi(const VDom &, const float *, float *, int steps, int strips, cudaStream_t) {
+    return logged("multi " + num(steps) + " strips " + num(strips));
+}
+cudaError_t multi_strips(const VDom &, int steps, int, int *strips) {
+    *strips = 10 * steps;
+    return logged("strips " + num(steps));
 }
 cudaError_t launch_step_cluster(int, const VDom &, const float *, float *, int n, Launch, bool pairs, cudaStream_t) {
     return logged("cluster " + num(n) + (pairs ? " pairs" : ""));

@@ -119,3 +119,20 @@ def test_autotune_tries_the_tile_that_fits_the_rows(lib, nx, warps):
     assert h("autotune", None) == 0
     tried = {tuple(s.split()[2:]) for s in h.log() if s.startswith("step 1 kind 6")}
     assert [t[3] for t in tried if t[5] == "2"] == [str(warps)], tried
+
+
+def test_strips_are_chosen_when_the_shape_is_set(lib):
+    """The search over strip counts is not part of a step, of whatever length."""
+    h = Handle(lib)
+    for k in (2, 3, 4):
+        assert h("set_launch", ctypes.byref(_CLaunch(2, 4, k, 9, 0))) == 0
+        assert h.log() == ["strips %d" % n for n in range(2, k + 1)]
+        for call in (("step", 131), ("step", 5), ("step", 2), ("step_monitored", 20, 10, FAKE, FAKE, FAKE)):
+            assert h(*call) == 0
+            lines = h.log()
+            assert not [s for s in lines if s.startswith("strips")]
+            assert all(s == "multi %d strips %d0" % (int(s[6]), int(s[6])) for s in lines if s.startswith("multi"))
+    assert h("autotune", None) == 0
+    h.log()
+    assert h("step", 131) == 0
+    assert not [s for s in h.log() if s.startswith("strips")]
