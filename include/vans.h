@@ -125,7 +125,8 @@ typedef struct {
  *         rows with all the steps as a wave, the populations in between held on
  *         chip, so that a launch moves the bytes of one step.  cpt 2, warps 4;
  *         ctas 0..2: strips for that many CTAs per SM (0: as many as fit).  A run
- *         of n steps is split into launches of equal size or one step apart; a
+ *         of n steps is split into launches of equal size or one step apart, none
+ *         of one step (but the last of an odd run of a batch with rows = 2); a
  *         single step (vans_step(h, 1), vans_step_raw, the forward steps of
  *         vans_adjoint_segment, a slab) is a launch of the single-step kind that
  *         vans_autotune found fastest (kind 0 after vans_set_launch).  Not for
@@ -200,7 +201,15 @@ int vans_update_eps(vans_t h, const float *eps_dev);
 /* ----------------------------------------------------------- time step -- */
 
 /* Advance the current state by nsteps >= 0 steps of the final LBE with P_i and
- * F_i.  Long runs replay a captured CUDA graph.  Errors: VANS_ERR_STATE before
+ * F_i.  Long runs replay a captured CUDA graph.  With kinds 0 to 7 the result has
+ * the same bits however the steps are split into calls.  Kind 8 (D2Q9) and kind 9
+ * round otherwise than those and than vans_step_raw: kind 8 the same for every
+ * split, kind 9 the same for every split into calls of two or more steps, while a
+ * step asked for alone is a single-step launch.  vans_autotune picks by time, so
+ * where two kinds are close its pick, and with it the last bits, may differ from
+ * run to run: a program that needs the same bits sets its launch
+ * (vans_set_launch).  States that vans_adjoint_segment is to recompute bit for bit
+ * are stepped by vans_step_single.  Errors: VANS_ERR_STATE before
  * vans_set_eps, VANS_ERR_ARG for nsteps < 0, VANS_ERR_CUDA. */
 int vans_step(vans_t h, int nsteps);
 

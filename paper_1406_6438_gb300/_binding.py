@@ -344,6 +344,9 @@ class Solver:
                "vans_update_eps")
 
     def step(self, nsteps: int = 1):
+        """nsteps steps.  With launch kind 9 a step asked for alone rounds otherwise than
+        one of a longer call (include/vans.h); states for ``adjoint_segment`` are
+        stepped by ``step_single``."""
         _check(self.lib.vans_step(self._h, int(nsteps)), "vans_step")
 
     def step_single(self, nsteps: int = 1):

@@ -174,7 +174,7 @@ struct vans_s {
     Launch Ls{4, 4, 1, 0};                      // single steps: L, or its stand-in if L is kind 9
     cudaGraphExec_t gexec[kGraphSizes] = {};   // 64, 32, ..., 2 single-step launches
     cudaGraphExec_t gmulti[kGraphSizes] = {};  // as many kind 9 launches of L.rows steps
-    int strips[vans::kMultiMax + 1] = {};       // of a kind 9 launch of 2..L.rows steps
+    int strips[vans::kMultiMax + 1] = {};       // of a kind 9 launch of 2, 3, ..L.rows steps
     int *flag = nullptr;                        // device status words (workspace)
     int *flag_host = nullptr;                   // pinned copy of flag[0] (vans_update_eps)
     cudaEvent_t flag_read = nullptr;            // behind that copy
@@ -249,7 +249,7 @@ Launch single_default(int q) { return q == 9 ? Launch{4, 4, 1, 0} : Launch{2, 4,
 // the strips of the kind 9 launches of L
 int set_strips(vans_t h, const Launch &L) {
     int n[vans::kMultiMax + 1] = {};
-    for (int k = 2; k <= L.rows; ++k)
+    for (int k = 2; k <= std::max(3, L.rows); ++k)
         if (vans::multi_strips(h->dom, k, L.ctas, &n[k]) != cudaSuccess) return VANS_ERR_CUDA;
     std::copy(std::begin(n), std::end(n), h->strips);
     return VANS_OK;
@@ -366,13 +366,21 @@ int run_single(vans_t h, int nsteps) {
 // The launches of nsteps steps (kind 8 apart).  Kind 9 takes up to L.rows steps per
 // launch: as few launches as that allows, of equal size or one step apart (9 steps at 4
 // per launch run as 3 + 3 + 3, not 4 + 4 + 1: a launch of fewer steps saves less than it
-// loses), the longer ones first.  A single step is a single-step launch.
+// loses), the longer ones first.  A step asked for alone is a single-step launch, which
+// rounds otherwise; a run of more leaves none alone (5 steps at 2 per launch run as 3 + 2;
+// but in a batch, whose table for 2 steps takes no third), so that its result does not
+// depend on how it was split into calls.
 void split_steps(vans_t h, int nsteps, Part p[2]) {
     p[0] = Part{nsteps, 1, h->gexec};
     p[1] = Part{0, 1, nullptr};
     if (h->L.kind != 9 || h->slab || nsteps < 2) return;
     const int most = h->L.rows, launches = 1 + (nsteps - 1) / most;
     const int few = nsteps / launches, longer = nsteps - few * launches;
+    if (few == 1 && !h->batched && nsteps > 2) {
+        p[0] = Part{1, 3, nullptr};
+        p[1] = Part{(nsteps - 3) / 2, 2, h->gmulti};
+        return;
+    }
     p[0] = Part{longer, few + 1, few + 1 == most ? h->gmulti : nullptr};
     p[1] = Part{launches - longer, few, few == most ? h->gmulti : nullptr};
 }

@@ -63,6 +63,24 @@ def test_result_does_not_depend_on_the_launch(walls):
         assert torch.equal(f, out[0])
 
 
+@pytest.mark.parametrize("walls", [False, True])
+def test_result_does_not_depend_on_calls_of_two_steps_or_more(walls):
+    """The same for odd counts: 11 steps in one call or in calls of at least two."""
+    torch = torch_cuda()
+    p, eps, f0 = _case(50, 150, walls, walls, 0, seed=4)
+    out = []
+    for L in LAUNCHES:
+        for calls in ((11,), (2, 9), (3, 3, 5), (7, 4)):
+            s = solver(p, eps, L)
+            s.set_populations(torch.from_numpy(f0).cuda())
+            for n in calls:
+                s.step(n)
+            out.append(s.populations())
+            s.close()
+    for f in out[1:]:
+        assert torch.equal(f, out[0])
+
+
 def test_single_steps_and_refusals():
     """vans_step(h, 1), step_raw and step_single run the single-step launch; plates
     on nodes, D3Q19 and shapes that are not built are refused."""

@@ -126,7 +126,7 @@ def test_strips_are_chosen_when_the_shape_is_set(lib):
     h = Handle(lib)
     for k in (2, 3, 4):
         assert h("set_launch", ctypes.byref(_CLaunch(2, 4, k, 9, 0))) == 0
-        assert h.log() == ["strips %d" % n for n in range(2, k + 1)]
+        assert h.log() == ["strips %d" % n for n in range(2, max(3, k) + 1)]
         for call in (("step", 131), ("step", 5), ("step", 2), ("step_monitored", 20, 10, FAKE, FAKE, FAKE)):
             assert h(*call) == 0
             lines = h.log()
@@ -136,3 +136,17 @@ def test_strips_are_chosen_when_the_shape_is_set(lib):
     h.log()
     assert h("step", 131) == 0
     assert not [s for s in h.log() if s.startswith("strips")]
+
+
+@pytest.mark.parametrize("launch", KINDS[1:])
+@pytest.mark.parametrize("n", [2, 3, 4, 5, 7, 9, 10, 11, 131])
+def test_no_step_is_left_alone(lib, launch, n):
+    """A run of two or more steps issues launches of several steps only: a single-step
+    launch rounds otherwise, and the result would depend on how the run was split."""
+    h = Handle(lib, launch)
+    for call in (("step", n), ("step_monitored", 3 * n + 3, n + 1, FAKE, FAKE, FAKE)):
+        assert h(*call) == 0
+        lines = [s for s in h.log() if s.startswith(("step", "multi"))]
+        if call[0] == "step_monitored":
+            lines = lines[:-1]              # the last emission's step has none after it
+        assert lines and all(s.startswith("multi") for s in lines)
