@@ -23,6 +23,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -54,19 +55,25 @@ TRAFFIC = {
     # dram__bytes_write.sum on the 4096^2 workload
     (4, 4, 3, 7, 2, "3df576119026cb61"): (677294336 + 561972480 + 677464320 + 560193536) // 2,
 }
-_PIPELINE_SOURCES = ("vans_step_tma.cu", "vans_pipeline.cuh", "vans_device.cuh", "vans_tma.cuh")
-KERNEL_SOURCES = {0: ("vans_step.cu", "vans_device.cuh")}
-KERNEL_SOURCES.update({k: _PIPELINE_SOURCES for k in (2, 4, 5, 6, 7)})
-KERNEL_SOURCES[8] = ("vans_cluster.cu", "vans_device.cuh")
-KERNEL_SOURCES[9] = ("vans_multi.cu", "vans_device.cuh")
+KERNEL_SOURCES = {0: "vans_step.cu", 8: "vans_cluster.cu", 9: "vans_multi.cu"}
+KERNEL_SOURCES.update({k: "vans_step_tma.cu" for k in (2, 4, 5, 6, 7)})
 
 
 def kernel_hash(kind: int = 2) -> str:
-    """Hash of the sources the step kernel of this launch kind is built from."""
-    h = hashlib.sha256()
-    for f in KERNEL_SOURCES[kind]:
-        with open(os.path.join(ROOT, "paper_1406_6438_gb300", "csrc", f), "rb") as fh:
-            h.update(fh.read())
+    """Hash of the source of this launch kind's step kernel and of the headers of this
+    repository that it includes, directly or through others."""
+    dirs = [os.path.join(ROOT, "paper_1406_6438_gb300", "csrc"), os.path.join(ROOT, "include")]
+    h, todo, seen = hashlib.sha256(), [KERNEL_SOURCES[kind]], set()
+    while todo:
+        name = todo.pop(0)
+        path = next(p for p in (os.path.join(d, name) for d in dirs) if os.path.exists(p))
+        with open(path, "rb") as fh:
+            text = fh.read()
+        h.update(text)
+        seen.add(name)
+        for inc in re.findall(rb'^#include "(.*)"', text, re.M):
+            if inc.decode() not in seen and inc.decode() not in todo:
+                todo.append(inc.decode())
     return h.hexdigest()[:16]
 
 
