@@ -39,10 +39,14 @@ METRIC = "MLUPS and % of HBM-bandwidth roofline; batched and adjoint MLUPS vs pl
 WORKLOAD = ("D2Q9 4096x4096 periodic, eps smoothed noise (sigma 16) in [0.4,1.0], tau 0.6, "
             "Ergun drag (d_p 21.33) + Forchheimer, body force along x, FP32 populations")
 BYTES_PER_CELL = {9: 9 * 4 * 2 + 4, 19: 19 * 4 * 2 + 4}     # algorithmic bytes per update
+# operations of the D2Q9 update of kind 9 (collide_rn of vans_pair.cuh; a multiply-add
+# counts two; the porosity terms, formed once per row and launch, are not counted)
+FLOPS_PER_CELL = 141
 # reverse step, D2Q9: lambda in and out (72), the state it reads (36), eps (4),
 # the compensated eps-gradient accumulators read and written (2 x 24)
 ADJ_BYTES_PER_CELL = 9 * 4 * 2 + 9 * 4 + 4 + 2 * 24
 FALLBACK_HBM_GBS = 6800.0
+SM_MAX_MHZ = 2070.0
 REPEATS = 5       # timed regions of K steps each; value = the median region
 E2E_JOBS = 6      # jobs of K steps in the end-to-end figure
 
@@ -93,6 +97,21 @@ def peaks():
         return float(d["hbm_gbs"]), "measured"
     except Exception:
         return FALLBACK_HBM_GBS, "fallback"
+
+
+def roofline(kind, cells, launch_s, steps_per_launch, sms):
+    """What the step kernel reaches of what bounds it: one step per launch HBM; kind 9, whose
+    launch reads and writes the state once for several steps, the FP32 pipe (rate of the
+    SMs' lanes at their highest clock), with its share of HBM beside it."""
+    peak, peak_kind = peaks()
+    gbs = BYTES_PER_CELL[9] * cells / launch_s / 1e9
+    hbm = {"achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak, "peak_kind": peak_kind}
+    if kind != 9:
+        return {"bound": "hbm", **hbm}
+    tflops = FLOPS_PER_CELL * cells * steps_per_launch / launch_s / 1e12
+    rate = sms * 128 * 2 * SM_MAX_MHZ * 1e6 / 1e12
+    return {"bound": "fp32", "achieved": tflops, "peak": rate, "unit": "TFLOP/s", "frac": tflops / rate,
+            "peak_kind": "SMs x 128 lanes x 2 x maximum clock", "flops_per_cell": FLOPS_PER_CELL, "hbm": hbm}
 
 
 # ------------------------------------------------------------------ clocks --
@@ -505,11 +524,8 @@ def main():
     t = statistics.median(regions)
     ok = sim.check()
     value = job_mlups(world, cells, args.steps, t)
-    # a launch reads and writes the state once, whatever number of steps it takes
-    # (kind 9 takes several and is bound by the FP32 pipe, not by HBM)
-    per_launch = t / launches
-    peak, peak_kind = peaks()
-    achieved = BYTES_PER_CELL[9] * cells / per_launch / 1e9
+    sms = torch.cuda.get_device_properties(local).multi_processor_count
+    roof = roofline(L.kind, cells, t / launches, args.steps / launches, sms)
     key = (L.cpt, L.warps, L.rows, L.kind, L.ctas, kernel_hash(L.kind))
     traffic = TRAFFIC.get(key) if args.n == 4096 else None
 
@@ -570,10 +586,8 @@ def main():
                    "parallelism": "replicas" if world > 1 else "single GPU",
                    "l2": "inputs larger than L2 (two 0.6 GB population buffers), no flush",
                    "launch": vars(L)},
-        "roofline": {"bound": "fp32" if L.kind == 9 else "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                     "frac": achieved / peak, "traffic": traffic,
-                     "peak_kind": peak_kind, "bytes_per_cell": BYTES_PER_CELL[9],
-                     "kernel": KERNEL_NAMES.get(L.kind, "?"), "launch_us": per_launch * 1e6,
+        "roofline": {**roof, "traffic": traffic, "bytes_per_cell": BYTES_PER_CELL[9],
+                     "kernel": KERNEL_NAMES.get(L.kind, "?"), "launch_us": t / launches * 1e6,
                      "steps_per_launch": args.steps / launches},
         "e2e": {"value": job_mlups(world, cells, E2E_JOBS * args.steps, t_e2e), "unit": "MLUPS",
                 "h2d_bytes_per_step": h2d / args.steps, "d2h_bytes_per_step": d2h / args.steps,

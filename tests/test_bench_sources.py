@@ -22,3 +22,19 @@ def test_hash_covers_every_header_of_the_kernel(tmp_path, monkeypatch, kind, hea
     with open(tmp_path / CSRC / header, "a") as f:
         f.write("\n// another\n")
     assert bench.kernel_hash(kind) != before
+
+
+def test_roofline_is_that_of_the_bound():
+    """Several steps per launch are bound by the FP32 pipe: their fraction is of its rate,
+    in TFLOP/s; one step per launch by HBM, in GB/s.  One step of 4096^2 in 200 us,
+    four in 400."""
+    cells = 4096 * 4096
+    r = bench.roofline(7, cells, 200e-6, 1, sms=152)
+    assert r["bound"] == "hbm" and r["unit"] == "GB/s" and r["achieved"] == pytest.approx(76 * cells / 200e-6 / 1e9)
+    assert r["frac"] == pytest.approx(r["achieved"] / bench.peaks()[0])
+    r = bench.roofline(9, cells, 400e-6, 4, sms=152)
+    assert r["bound"] == "fp32" and r["unit"] == "TFLOP/s"
+    assert r["achieved"] == pytest.approx(bench.FLOPS_PER_CELL * cells / 100e-6 / 1e12)
+    assert r["peak"] == pytest.approx(152 * 128 * 2 * 2.07e9 / 1e12, rel=0.02)
+    assert r["frac"] == pytest.approx(r["achieved"] / r["peak"]) and 0 < r["frac"] < 1
+    assert r["hbm"]["achieved"] == pytest.approx(76 * cells / 400e-6 / 1e9)
