@@ -114,6 +114,15 @@ def roofline(kind, cells, launch_s, steps_per_launch, sms):
             "peak_kind": "SMs x 128 lanes x 2 x maximum clock", "flops_per_cell": FLOPS_PER_CELL, "hbm": hbm}
 
 
+def load_balance(b, kind):
+    """The load balance of one more step with per-CTA timing records: the mean over the SMs
+    of their busy span / the step's makespan.  With kind 9 the profile is of the batch's
+    single-step launch, not of the launches that were timed; kind 0 has none."""
+    if kind == 0:
+        return {}
+    return {"single_step_load_balance" if kind == 9 else "load_balance": b.profile_step()}
+
+
 # ------------------------------------------------------------------ clocks --
 class ClockSampler:
     """nvidia-smi samples of SM clock and throttle reasons during a region."""
@@ -366,10 +375,7 @@ def bench_batched(torch, V, W, args=None):
            "gb_s": BYTES_PER_CELL[9] * cells * n / per_launch / t / 1e9,
            "launch": vars(L), "launches": b.launch_count - c0}
     out["frac_of_peak"] = out["gb_s"] / peaks()[0]
-    if L.kind != 0:
-        # one more step with per-CTA timing records: the load balance, mean over
-        # the SMs of their busy span / the step's makespan
-        out["load_balance"] = b.profile_step()
+    out.update(load_balance(b, L.kind))
     b.close()
     return out
 

@@ -38,3 +38,14 @@ def test_roofline_is_that_of_the_bound():
     assert r["peak"] == pytest.approx(152 * 128 * 2 * 2.07e9 / 1e12, rel=0.02)
     assert r["frac"] == pytest.approx(r["achieved"] / r["peak"]) and 0 < r["frac"] < 1
     assert r["hbm"]["achieved"] == pytest.approx(76 * cells / 400e-6 / 1e9)
+
+
+@pytest.mark.parametrize("kind,key", [(4, "load_balance"), (9, "single_step_load_balance"), (0, None)])
+def test_load_balance_names_the_launch_it_is_of(kind, key):
+    """The profile of a batch that runs several steps per launch is of its single-step
+    launch, which the timed region does not run."""
+    class Batch:
+        def profile_step(self):
+            return {"efficiency": 0.9}
+    got = bench.load_balance(Batch(), kind)
+    assert got == ({} if key is None else {key: {"efficiency": 0.9}})
