@@ -39,7 +39,7 @@ METRIC = "MLUPS and % of HBM-bandwidth roofline; batched and adjoint MLUPS vs pl
 WORKLOAD = ("D2Q9 4096x4096 periodic, eps smoothed noise (sigma 16) in [0.4,1.0], tau 0.6, "
             "Ergun drag (d_p 21.33) + Forchheimer, body force along x, FP32 populations")
 BYTES_PER_CELL = {9: 9 * 4 * 2 + 4, 19: 19 * 4 * 2 + 4}     # algorithmic bytes per update
-# operations of the D2Q9 update of kind 9 (collide_rn of vans_pair.cuh; a multiply-add
+# operations of the D2Q9 update of kind 9 (collide_pair of vans_pair.cuh; a multiply-add
 # counts two; the porosity terms, formed once per row and launch, are not counted)
 FLOPS_PER_CELL = 141
 # reverse step, D2Q9: lambda in and out (72), the state it reads (36), eps (4),

@@ -225,21 +225,16 @@ __global__ void __launch_bounds__(256) k_step(const VDom d, const float *__restr
     if (EMIT && blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) atomicAdd(&mon.stats[3], 1.f);
 }
 
-template <int Q, int CPT, bool EDGE, bool EMIT>
+template <int CPT, bool EDGE, bool EMIT>
 __device__ __forceinline__ void moments_row(const VDom &d, const float *__restrict__ fin, const Monitor &mon,
-                                            bool whole, int y, int z, int x0, int lane) {
+                                            bool whole, int y, int x0, int lane) {
+    constexpr int Q = 9;
     using L = Lat<Q>;
     const Nb3 Y = nb3<EDGE>(y, d.ny, d.wall_y);
-    Nb3 Z;
-    if (Q == 19) {
-        Z = nb3<EDGE>(z, d.nz, d.wall_z);
-    } else {
-        Z.r[0] = Z.r[1] = Z.r[2] = 0;
-        Z.wall[0] = Z.wall[1] = Z.wall[2] = false;
-    }
+    const Nb3 Z = {};
     float h[Q][CPT], E[3][3][CPT + 2];
-    load_row<Q, CPT>(d, fin, Y, Z, y, z, x0, lane, h, E);
-    const long long n = ((long long)z * d.ny + y) * d.nx + x0;
+    load_row<Q, CPT>(d, fin, Y, Z, y, 0, x0, lane, h, E);
+    const long long n = (long long)y * d.nx + x0;
     // whole: every row of the dense outputs starts on a vector boundary
     auto put = [&](float *p, const float v[CPT]) {
         if (whole && x0 + CPT <= d.nx) {
@@ -275,8 +270,7 @@ __device__ __forceinline__ void moments_row(const VDom &d, const float *__restri
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             hh[i] = h[i][k];
-            const bool wall = Y.wall[1 + L::ey(i)] || Z.wall[1 + L::ez(i)];
-            et[i] = (i == 0 || wall) ? e0 : E[1 + L::ey(i)][1 + L::ez(i)][k + 1 + L::ex(i)];
+            et[i] = (i == 0 || Y.wall[1 + L::ey(i)]) ? e0 : E[1 + L::ey(i)][1][k + 1 + L::ex(i)];
         }
         if (EDGE) apply_moving_wall<Q>(d, Y.wall[2], Z, e0, hh);
         Macro<Q> M;
@@ -302,14 +296,14 @@ __device__ __forceinline__ void moments_row(const VDom &d, const float *__restri
     if (EMIT) emit_maxima(mon, lane, dmax, umax, bad);
 }
 
-// rho and u of the state (Eqs. 0moment and 1moment), and with EMIT the reductions of
+// rho and u of a D2Q9 state (Eqs. 0moment and 1moment), and with EMIT the reductions of
 // a monitoring emission.  Bound by the loads in flight: rows by vector loads (4 cells
 // per lane) with as many blocks per SM as the registers allow without spills, 7 (6 with
 // EMIT): 4096^2 245 -> 158 us (0.82 of the copy bandwidth), 2048^2 68 -> 47, 1501 x 733
 // 20.4 -> 13.1, against one cell per thread.  D3Q19 keeps that form (vans_aux.cu): 2
 // cells per lane measured the same at 256 x 256 x 128 and 64 us instead of 48 at
 // 150 x 110 x 90.
-template <int Q, int CPT, bool EMIT>
+template <int CPT, bool EMIT>
 __global__ void __launch_bounds__(128, EMIT ? 6 : 7) k_moments_rows(const VDom d, const float *__restrict__ fin, int nxb,
                                                       const Monitor mon, bool whole) {
     pdl_trigger();
@@ -318,12 +312,10 @@ __global__ void __launch_bounds__(128, EMIT ? 6 : 7) k_moments_rows(const VDom d
     const int bx = blockIdx.x % nxb, r = (blockIdx.x / nxb) * blockDim.y + threadIdx.y;
     const int xw = (bx * (blockDim.x >> 5) + wx) * 32 * CPT;
     if (r >= d.rows || xw >= d.nx) return;                 // whole warp
-    const int y = r % d.ny, z = r / d.ny;
-    const bool edge = (y == 0) || (y == d.ny - 1) || (Q == 19 && (z == 0 || z == d.nz - 1));
-    if (edge)
-        moments_row<Q, CPT, true, EMIT>(d, fin, mon, whole, y, z, xw + lane * CPT, lane);
+    if (r == 0 || r == d.ny - 1)
+        moments_row<CPT, true, EMIT>(d, fin, mon, whole, r, xw + lane * CPT, lane);
     else
-        moments_row<Q, CPT, false, EMIT>(d, fin, mon, whole, y, z, xw + lane * CPT, lane);
+        moments_row<CPT, false, EMIT>(d, fin, mon, whole, r, xw + lane * CPT, lane);
     if (EMIT && blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) atomicAdd(&mon.stats[3], 1.f);
 }
 
@@ -407,7 +399,7 @@ cudaError_t launch_step_monitor(int q, const VDom &d, const float *fin, float *f
     return cudaGetLastError();
 }
 
-template <int Q, int CPT, bool EMIT>
+template <int CPT, bool EMIT>
 static cudaError_t launch_moments_t(const VDom &d, const float *state, const Monitor &mon,
                                     cudaStream_t stream) {
     const int warps = std::min(4, (d.nx + 32 * CPT - 1) / (32 * CPT)), rows = 4 / warps;
@@ -415,7 +407,7 @@ static cudaError_t launch_moments_t(const VDom &d, const float *state, const Mon
     const long long nblocks = (long long)nxb * ((d.rows + rows - 1) / rows);
     if (nblocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     const bool whole = d.nx % CPT == 0 && ((uintptr_t)mon.rho | (uintptr_t)mon.u) % (4 * CPT) == 0;
-    return launch_pdl(k_moments_rows<Q, CPT, EMIT>, dim3((unsigned)nblocks), dim3(32 * warps, rows), 0, stream,
+    return launch_pdl(k_moments_rows<CPT, EMIT>, dim3((unsigned)nblocks), dim3(32 * warps, rows), 0, stream,
                       d, state, nxb, mon, whole);
 }
 
@@ -423,8 +415,8 @@ cudaError_t launch_moments_rows(const VDom &d, const float *state, float *rho, f
                                 float *stats, float *part, cudaStream_t stream) {
     const Monitor mon{rho, u, stats, part};
     if (d.q != 9) return cudaErrorInvalidValue;
-    return stats ? launch_moments_t<9, 4, true>(d, state, mon, stream)
-                 : launch_moments_t<9, 4, false>(d, state, mon, stream);
+    return stats ? launch_moments_t<4, true>(d, state, mon, stream)
+                 : launch_moments_t<4, false>(d, state, mon, stream);
 }
 
 // stats[c] = max over the slots of part[c][slot], c = 0..2 (one block)
