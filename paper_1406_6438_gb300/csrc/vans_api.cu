@@ -90,7 +90,7 @@ bool launch_ok(const vans_launch *c, int q, bool batched) {
     if (c->kind == 8)       // cluster-resident steps: cluster of up to `rows` CTAs
         return !batched && c->cpt == 1 && c->ctas == 0 && (c->warps == 8 || c->warps == 16) &&
                c->rows >= 2 && c->rows <= 16;
-    if (c->kind == 9)       // `rows` steps per launch held in registers
+    if (c->kind == 9)       // `rows` steps per launch, held on chip
         return q == 9 && c->cpt == 2 && c->warps == vans::kMultiWarps && c->rows >= 2 &&
                c->rows <= vans::kMultiMax && c->ctas <= 2;
     // kinds 1 and 3 are not built (never the fastest at any measured size)
@@ -294,31 +294,11 @@ struct Part {
     cudaGraphExec_t *gs;
 };
 
-// launches of `p` that go out by themselves before its graphs, which start at parity 0
-int ahead_of_graphs(const Part &p, int par) { return p.gs && p.count >= 2 && par != 0 ? 1 : 0; }
-
-// Captures the graphs that `p` will replay; par: the parity it starts from, on return
-// the one it ends with.  A size is captured when a run first needs it (all six at once
-// are 126 launches, of which a short run replays a few), and before any step of that
-// run is issued, so that a capture that fails leaves the state as it was.
-int capture_for(vans_t h, const Part &p, int &par) {
-    int left = p.count - ahead_of_graphs(p, par);
-    par ^= p.count & 1;
-    for (int k = 0; p.gs && left >= 2 && k < kGraphSizes; ++k) {
-        const int n = kGraphSteps >> k;
-        if (left < n) continue;
-        left %= n;
-        if (p.gs[k]) continue;
-        const int rc = capture_launches(h, n, p.steps, &p.gs[k]);
-        if (rc) {
-            drop_graph(h);
-            return rc;
-        }
-    }
-    return VANS_OK;
-}
-
-// Issues the launches of `p`; the parity lives in h->cur (single) or h->parity (batched)
+// Issues the launches of `p`; the parity lives in h->cur (single) or h->parity (batched).
+// A graph size is captured when a run first needs it: all six at once are 126 launches,
+// of which a short run replays a few, and the GPU runs the larger ones' replays while the
+// smaller are captured.  Where a size cannot be captured the rest of the run is launched
+// one by one, so that no run ends half done for the want of a graph.
 int run_launches(vans_t h, const Part &p) {
     int &par = h->batched ? h->parity : h->cur;
     int left = p.count;
@@ -328,13 +308,24 @@ int run_launches(vans_t h, const Part &p) {
         --left;
         return VANS_OK;
     };
-    if (ahead_of_graphs(p, par))
+    bool graphs = p.gs && left >= 2;
+    if (graphs && par != 0)             // graphs start at parity 0
         if (const int rc = one()) return rc;
-    for (int k = 0; p.gs && left >= 2 && k < kGraphSizes; ++k) {
+    for (int k = 0; graphs && k < kGraphSizes; ++k) {
         const int n = kGraphSteps >> k;
-        for (; left >= n; left -= n) {
+        while (left >= n) {
+            if (!p.gs[k] && capture_launches(h, n, p.steps, &p.gs[k]) != VANS_OK) {
+                cudaStreamCaptureStatus user = cudaStreamCaptureStatusNone;
+                if (cudaStreamIsCapturing(h->stream, &user) != cudaSuccess ||
+                    user != cudaStreamCaptureStatusNone)
+                    return VANS_ERR_CUDA;            // (a captured stream takes no graph either)
+                cudaGetLastError();                  // not the next launch's error
+                graphs = false;
+                break;
+            }
             if (cudaGraphLaunch(p.gs[k], h->stream) != cudaSuccess) return VANS_ERR_CUDA;
             h->launches += n;
+            left -= n;
         }
     }
     while (left > 0)
@@ -357,10 +348,7 @@ int run_cluster(vans_t h, int nsteps, const Launch &L, bool pairs) {
 // that rounds like them: the forward run of a reverse pass
 int run_single(vans_t h, int nsteps) {
     if (!h->batched && h->Ls.kind == 8 && nsteps > 0) return run_cluster(h, nsteps, h->Ls, false);
-    const Part p{nsteps, 1, h->gexec};
-    int par = h->batched ? h->parity : h->cur;
-    const int rc = capture_for(h, p, par);
-    return rc ? rc : run_launches(h, p);
+    return run_launches(h, Part{nsteps, 1, h->gexec});
 }
 
 // The launches of nsteps steps (kind 8 apart).  Kind 9 takes up to L.rows steps per
@@ -385,31 +373,12 @@ void split_steps(vans_t h, int nsteps, Part p[2]) {
     p[1] = Part{launches - longer, few, few == most ? h->gmulti : nullptr};
 }
 
-// the graphs of run_steps(h, nsteps) from parity par, which becomes the one after it
-int prepare_steps(vans_t h, int nsteps, int &par) {
-    if (!h->batched && h->L.kind == 8) {
-        par ^= nsteps & 1;
-        return VANS_OK;
-    }
-    Part p[2];
-    split_steps(h, nsteps, p);
-    const int rc = capture_for(h, p[0], par);
-    return rc ? rc : capture_for(h, p[1], par);
-}
-
-// nsteps steps, whose graphs prepare_steps has made
-int issue_steps(vans_t h, int nsteps) {
+int run_steps(vans_t h, int nsteps) {
     if (!h->batched && h->L.kind == 8 && nsteps > 0) return run_cluster(h, nsteps, h->L, true);
     Part p[2];
     split_steps(h, nsteps, p);
     const int rc = run_launches(h, p[0]);
     return rc ? rc : run_launches(h, p[1]);
-}
-
-int run_steps(vans_t h, int nsteps) {
-    int par = h->batched ? h->parity : h->cur;
-    const int rc = prepare_steps(h, nsteps, par);
-    return rc ? rc : issue_steps(h, nsteps);
 }
 
 int make_streams(vans_t h, void *stream) {
@@ -817,24 +786,20 @@ int vans_step_monitored(vans_t h, int nsteps, int every, float *rho_dev, float *
         return VANS_ERR_ARG;
     if (h->dom.nee || h->slab) return VANS_ERR_UNSUPPORTED;    // plates on nodes: use vans_moments
     if (!h->eps_set) return VANS_ERR_STATE;
+    if (cudaMemsetAsync(stats_dev, 0, 4 * sizeof(float), h->stream) != cudaSuccess ||
+        cudaMemsetAsync(h->mon_part, 0, kMonFloats * sizeof(float), h->stream) != cudaSuccess)
+        return VANS_ERR_CUDA;
     // An emission reads the state before the step that it stands for.  With several
     // steps per launch that step goes with the plain ones up to the next emission
     // (2048^2: 62 us for the emission and 27 for the step, in one kernel 111); single
     // steps emit themselves (4096^2: 420 us, 215 + 250 apart).
     const bool fused = h->L.kind != 9 || every == 1;
-    // plain steps before the emission that follows step `done`, the owed one included
-    auto plain = [&](int done) { return std::min(every - 1, nsteps - done - 1) + (!fused && done > 0); };
-    for (int done = 0, par = h->cur; done < nsteps; done += std::min(every, nsteps - done)) {
-        const int rc = prepare_steps(h, plain(done), par);
+    int done = 0, owed = 0;
+    while (done < nsteps) {
+        const int plain = std::min(every - 1, nsteps - done - 1);
+        const int rc = run_steps(h, owed + plain);
         if (rc) return rc;
-        if (fused) par ^= 1;
-    }
-    if (cudaMemsetAsync(stats_dev, 0, 4 * sizeof(float), h->stream) != cudaSuccess ||
-        cudaMemsetAsync(h->mon_part, 0, kMonFloats * sizeof(float), h->stream) != cudaSuccess)
-        return VANS_ERR_CUDA;
-    for (int done = 0; done < nsteps; done += std::min(every, nsteps - done)) {
-        const int rc = issue_steps(h, plain(done));
-        if (rc) return rc;
+        done += plain + 1;
         ++h->launches;
         const float *in = h->st[h->cur];
         if ((fused ? vans::launch_step_monitor(h->q, h->dom, in, h->st[h->cur ^ 1], rho_dev, u_dev, stats_dev,
@@ -843,11 +808,10 @@ int vans_step_monitored(vans_t h, int nsteps, int every, float *rho_dev, float *
                                                h->stream)) != cudaSuccess)
             return VANS_ERR_CUDA;
         if (fused) h->cur ^= 1;
+        else owed = 1;
     }
-    if (!fused && nsteps > 0) {
-        const int rc = run_steps(h, 1);
-        if (rc) return rc;
-    }
+    const int rc = run_steps(h, owed);
+    if (rc) return rc;
     if (nsteps > 0) {
         ++h->launches;
         if (vans::launch_monitor_finalize(h->mon_part, stats_dev, h->stream) != cudaSuccess)

@@ -11,6 +11,7 @@ namespace {
 
 std::vector<std::string> g_log, *g_into = &g_log;   // the capture's list while one is open
 std::map<std::string, int> g_fail;                  // calls until this one fails (1: the next)
+cudaError_t g_last = cudaSuccess;                   // as cudaGetLastError has it
 std::vector<std::vector<std::string>> g_graphs;
 std::string g_text;
 bool g_user_capture = false, g_quiet = false;       // quiet: steps are counted, not logged
@@ -26,12 +27,13 @@ void put(const std::string &s) {
 }
 cudaError_t call(const char *name) {
     auto f = g_fail.find(name);
-    if (f != g_fail.end() && f->second > 0 && --f->second == 0) return cudaErrorUnknown;
+    if (f != g_fail.end() && f->second > 0 && --f->second == 0) return g_last = cudaErrorUnknown;
     return cudaSuccess;
 }
-cudaError_t logged(const std::string &s) {
+cudaError_t logged(const std::string &s) {          // as a launch: an earlier call's error too
     put(s);
-    return call(s.substr(0, s.find(' ')).c_str());
+    call(s.substr(0, s.find(' ')).c_str());
+    return cudaGetLastError();
 }
 std::string num(long long v) { return std::to_string(v); }
 
@@ -44,6 +46,7 @@ void fake_reset() {
     g_fail.clear();
     g_into = &g_log;
     g_user_capture = g_quiet = false;
+    g_last = cudaSuccess;
     g_steps = 0;
 }
 void fake_quiet() { g_quiet = true; }
@@ -58,7 +61,11 @@ const char *fake_log() {
 
 cudaError_t cudaGetDevice(int *d) { *d = 0; return cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr, int) { *v = 152; return cudaSuccess; }
-cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaGetLastError() {
+    const cudaError_t e = g_last;
+    g_last = cudaSuccess;
+    return e;
+}
 cudaError_t cudaEventCreate(cudaEvent_t *e) { *e = (cudaEvent_t)8; return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { *e = (cudaEvent_t)8; return call("event"); }
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
@@ -96,6 +103,7 @@ cudaError_t cudaGraphInstantiate(cudaGraphExec_t *e, cudaGraph_t g, unsigned lon
 cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
 cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
 cudaError_t cudaGraphLaunch(cudaGraphExec_t e, cudaStream_t) {
+    if (g_user_capture) return cudaErrorStreamCaptureUnsupported;
     g_steps += g_graph_steps[(size_t)e - 1];
     if (!g_quiet)
         for (const auto &s : g_graphs[(size_t)e - 1]) g_log.push_back(s);

@@ -61,21 +61,37 @@ KINDS = [(4, 4, 1, 0, 0), (2, 4, 4, 9, 0), (2, 4, 3, 9, 0), (2, 4, 2, 9, 0)]
 @pytest.mark.parametrize("launch", KINDS)
 @pytest.mark.parametrize("what", ["capture", "instantiate"])
 @pytest.mark.parametrize("nth", [1, 2])
-def test_a_failed_capture_runs_no_step(lib, launch, what, nth):
-    """Graphs of several sizes serve a run: where one of them cannot be made, none of the
-    run's steps has been issued, and the run can be asked for again."""
+def test_a_failed_capture_ends_no_run_half_done(lib, launch, what, nth):
+    """Graphs of several sizes serve a run: where one of them cannot be made, the run takes
+    its steps all the same, and the next one captures again."""
     for warm in (0, 1):
         h = Handle(lib, launch)
         h("step", warm)
         h.log()
-        for call in (("step", 63 * launch[2]), ("step_monitored", 190, 63, FAKE, FAKE, FAKE)):
+        for n, call in ((63 * launch[2], ("step", 63 * launch[2])), (190, ("step_monitored", 190, 63, FAKE, FAKE, FAKE))):
             h.log()
             lib.fake_fail(what.encode(), nth)
-            assert h(*call) == ERR_CUDA
-            assert h.steps() == 0
-            assert h("step", 0) == 0 and h.steps() == 0
+            assert h(*call) == 0
+            # (kind 9 emits between launches of several steps, which then are all of the steps)
+            assert h.steps() == n
         assert h("step", 63 * launch[2]) == 0
         assert h.steps() == 63 * launch[2]
+
+
+@pytest.mark.parametrize("launch", KINDS)
+def test_a_captured_stream_takes_no_run_that_needs_graphs(lib, launch):
+    """Refused with nothing recorded, whether its graphs exist, are made or cannot be."""
+    for warm in (False, True):
+        for fails in (False, True):
+            h = Handle(lib, launch)
+            if warm:
+                h("step", 64 * launch[2])
+                h.log()
+            if fails:
+                lib.fake_fail(b"capture", 1)
+            lib.fake_user_capture(1)
+            assert h("step", 64 * launch[2]) == ERR_CUDA
+            assert h.steps() == 0
 
 
 @pytest.mark.parametrize("launch", KINDS)
