@@ -153,6 +153,7 @@ void fill_dom(const vans_params *p, VDom &d) {
         d.cb = (float)(1.75 / sqrt(150.0 * p->K));
     }
     d.cells = (long long)p->nx * p->ny * p->nz;
+    d.tails = row_tails(p->q, p->nx, d.cells);
     d.uw[0] = p->u_wall[0];
     d.uw[1] = p->u_wall[1];
     d.uw[2] = (p->q == 19) ? p->u_wall[2] : 0.f;

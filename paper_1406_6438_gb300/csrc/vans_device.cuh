@@ -222,12 +222,12 @@ __device__ __forceinline__ void store_halo_hi(float *row, int nx, float v) {
 
 // The rest of the sector that column nx - 1 lies in, as zeros, by the lanes of columns
 // x >= nx: in part written, that sector too costs a DRAM read per direction and row
-// (250^3, one cell per thread: 432 -> 392 us; domains within L2 lose up to 3 %; with
-// the zeros selected in the lanes' ordinary stores 409).  Column nx of the directions
-// moving -x is the halo copy.
-template <int Q>
-__device__ __forceinline__ bool in_row_tail(int nx, int x) {
-    return Q == 19 && x >= nx && x < ((nx + 7) & ~7);
+// (250^3, one cell per thread: 418 -> 391 us; with the zeros selected in the lanes'
+// ordinary stores 409).  Where it pays: row_tails (vans_internal.h).  Column nx of the
+// directions moving -x is the halo copy.
+template <int Q, int TW>
+__device__ __forceinline__ bool in_row_tail(const VDom &d, int x) {
+    return Q == 19 && (d.tails >> (TW / 32) & 1) && x >= d.nx && x < ((d.nx + 7) & ~7);
 }
 template <int Q>
 __device__ __forceinline__ void store_row_tail(float *fout, long long plane, long long ro, int nx, int x) {

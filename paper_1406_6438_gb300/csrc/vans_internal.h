@@ -38,6 +38,7 @@ struct VDom {
     int moving;           // 1: the upper y wall moves with velocity uw (bounce-back walls)
     float uw[3];          // velocity of the upper y wall / plate
     int nee;              // 1: rows 0 and ny-1 are plate nodes (non-equilibrium extrapolation)
+    int tails;            // row_tails: the tile widths that store a row's last sector whole
 };
 
 // One tile of the batched register-load kernel: a block-sized piece of one
@@ -80,6 +81,18 @@ inline int col0_for(int q) { return q == 19 ? 32 : 8; }
 // Floats per padded row for a row of nx cells: column 0 at col0_for(q),
 // columns -1 and nx as halo copies, rounded up to whole 128-byte lines.
 int pitch_for(int q, int nx);
+// D3Q19: bit k set where a step in tiles of 32 k cells stores the last sector of a row
+// whole (in_row_tail).  That spares a DRAM read, so both states have to lie beyond the
+// L2 (152 bytes per cell; within it the stores cost up to 5 %: 35^3 5.3 -> 5.6 us, 90^3
+// 24.6 -> 25.4) and the lanes to be in use, which a step of idle lanes waits for instead
+// (tiles of 256 cells, two per thread: rows of 221 and 250 cells 167 -> 148 and 480 -> 461
+// us, rows of 150 cells 65.6 -> 70.2).
+inline int row_tails(int q, int nx, long long cells) {
+    int m = 0;
+    for (int k = 1; q == 19 && cells > 1000000 && k <= 8; ++k)
+        if (5LL * nx >= 4LL * (32 * k) * ((nx + 32 * k - 1) / (32 * k))) m |= 1 << k;
+    return m;
+}
 // The kernel descriptor of one domain from validated parameters: sizes, row
 // layout, relaxation and drag constants, walls.  Buffers (eps, f, status) are
 // left null for the caller to set.

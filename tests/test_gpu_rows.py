@@ -65,3 +65,28 @@ def test_the_narrowest_tile_takes_short_rows(nx):
     for stages in (2, 3):
         rho, u, f = gpu_run(p, eps, 5, f0, launch=Launch(1, 2, stages, 6))
         assert np.abs(f - f_o).max() <= 2e-7 and rel_u(u, u_o) <= 1e-5
+
+
+@pytest.mark.parametrize("shape", [(61, 67, 250), (64, 75, 221), (80, 100, 129)])
+def test_last_sectors_stored_whole_of_a_domain_beyond_the_l2(shape):
+    """More than a million cells, where tiles that a row fills to 4/5 store its last sector
+    whole: kind 6 leaves the bits of the register-load kernel, which stores cells and halo
+    copies alone, whoever steps next; the strip kinds agree within 2e-7."""
+    torch = torch_cuda()
+    nz, ny, nx = shape
+    p = W.params(q=19, nx=nx, ny=ny, nz=nz, wall_mask=2, tau=0.7, g=(3e-4, -1e-4, 2e-4), drag_mode=2, k_mode=0,
+                 d_p=6.0)
+    eps = W.smoothed_noise(shape, 2.0, 0.4, 1.0, nx)
+    plain, fit = Launch(1, 4, 1), Launch(1, (nx + 31) // 32, 2, 6)
+    out = []
+    for turn in ([plain] * 6, [fit] * 6, [fit, plain] * 3, [Launch(2, 4, 2, 2), Launch(1, 8, 2, 4)] * 3,
+                 [Launch(1, 4, 3, 4), fit] * 3):
+        s = solver(p, eps, turn[0])
+        for L in turn:
+            s.launch = L
+            s.step(1)
+        out.append(s.populations())
+        s.close()
+    assert torch.equal(out[1], out[0]) and torch.equal(out[2], out[0])
+    for f in out[3:]:
+        assert float((f - out[0]).abs().max()) <= 2e-7
