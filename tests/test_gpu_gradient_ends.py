@@ -186,3 +186,9 @@ def test_sums_that_leave_the_range_of_floats(q, shape, bits):
         assert np.array_equal(np.isnan(out), np.isnan(v)), kind
         ok = ~np.isnan(v)
         assert np.allclose(out[ok], v[ok], rtol=1e-5, atol=1e-30), kind
+
+
+@pytest.mark.parametrize("q,shape", [(9, (1, 256, 3)), (9, (1, 257, 3)), (19, (16, 16, 3)), (19, (17, 16, 3))])
+def test_flux_of_one_block_and_of_a_cluster(q, shape):
+    """At the most rows that one block sums and one row more."""
+    test_flux_is_the_sum_of_the_outlet(q, shape)
