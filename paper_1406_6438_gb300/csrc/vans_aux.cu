@@ -730,7 +730,11 @@ static int grid_for(long long n, int threads) {
 
 cudaError_t launch_moments(int q, const VDom &d, const float *state, float *rho, float *u,
                            cudaStream_t s) {
-    if (q == 9 && !d.nee) return launch_moments_rows(d, state, rho, u, nullptr, nullptr, s);
+    // by rows where these use at least 5/8 of the lanes (128 cells per warp): with fewer the
+    // idle lanes cost more than the vector loads save (3 M cells, rows of 9 cells 341 us
+    // against 79, 64 58 and 51, 80 49 and 50, 129 56 and 50, 160 47 and 50, 260 45 and 50)
+    if (q == 9 && !d.nee && 8LL * d.nx >= 5LL * 128 * ((d.nx + 127) / 128))
+        return launch_moments_rows(d, state, rho, u, nullptr, nullptr, s);
     const int g = grid_for(d.cells, 256);
     VANS_DISPATCH_Q(q, (k_moments<9><<<g, 256, 0, s>>>(d, state, rho, u)),
                     (k_moments<19><<<g, 256, 0, s>>>(d, state, rho, u)));
