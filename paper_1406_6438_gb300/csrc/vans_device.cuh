@@ -226,8 +226,8 @@ __device__ __forceinline__ void store_halo_hi(float *row, int nx, float v) {
 // ordinary stores 409).  Where it pays: row_tails (vans_internal.h).  Column nx of the
 // directions moving -x is the halo copy.
 template <int Q, int TW>
-__device__ __forceinline__ bool in_row_tail(const VDom &d, int x) {
-    return Q == 19 && (d.tails >> (TW / 32) & 1) && x >= d.nx && x < ((d.nx + 7) & ~7);
+__device__ __forceinline__ bool row_tails_on(const VDom &d) {
+    return Q == 19 && (d.tails >> (TW / 32) & 1);
 }
 template <int Q>
 __device__ __forceinline__ void store_row_tail(float *fout, long long plane, long long ro, int nx, int x) {

@@ -82,7 +82,7 @@ inline int col0_for(int q) { return q == 19 ? 32 : 8; }
 // columns -1 and nx as halo copies, rounded up to whole 128-byte lines.
 int pitch_for(int q, int nx);
 // D3Q19: bit k set where a step in tiles of 32 k cells stores the last sector of a row
-// whole (in_row_tail).  That spares a DRAM read, so both states have to lie beyond the
+// whole (store_row_tail).  That spares a DRAM read, so both states have to lie beyond the
 // L2 (152 bytes per cell; within it the stores cost up to 5 %: 35^3 5.3 -> 5.6 us, 90^3
 // 24.6 -> 25.4) and the lanes to be in use, which a step of idle lanes waits for instead
 // (tiles of 256 cells, two per thread: rows of 221 and 250 cells 167 -> 148 and 480 -> 461

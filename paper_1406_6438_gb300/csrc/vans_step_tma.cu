@@ -334,8 +334,13 @@ __device__ __forceinline__ void ring_tile(const VDom &d, const float *__restrict
                     for (int i = 0; i < Q; ++i)
                         if (L::ex(i) > 0) store_halo_lo<Q>(fout + i * d.plane + ro, o[i]);
                 }
-            } else if (in_row_tail<Q, NT * CPT>(d, x)) {
-                store_row_tail<Q>(fout, d.plane, ro, d.nx, x);
+            }
+        }
+        if (row_tails_on<Q, NT * CPT>(d)) {
+#pragma unroll
+            for (int cc = 0; cc < CPT; ++cc) {
+                const int x = xs + tid + cc * NT;
+                if (x >= d.nx && x < ((d.nx + 7) & ~7)) store_row_tail<Q>(fout, d.plane, ro, d.nx, x);
             }
         }
     }
