@@ -20,9 +20,10 @@
 // shared memory, the e_y > 0 values that wait two turns are kept there too (in
 // registers they cost 12 per step and as many moves), and the next row's loads go
 // out before the last step: 160-168 registers, 12 warps per SM, none spilled.
-// Measured at 4096^2 (us per step; ncu: DRAM 0.3 of its peak): T = 2 135, 3 107,
-// 4 101, periodic or between walls; 2048^2 27, 1024^2 8.4 (kind 7: 12.2), 512^2
-// 3.8 (kind 0: 4.9).  With 128 registers (16 warps) T = 2 gains 3 %, 3 and 4
+// Measured at 4096^2 (us per step; ncu: DRAM 0.3 of its peak): T = 2 135.6, 3 106.7,
+// 4 100.7, between walls 135.8, 108.0, 101.2; with the autotuner's shape 2048^2 27.0,
+// between walls 27.4, 1024^2 8.4 and 9.2 (kind 7: 12.1), 512^2
+// 3.8 and 4.4 (kind 0: 4.8).  With 128 registers (16 warps) T = 2 gains 3 %, 3 and 4
 // spill and lose.
 //
 // The result does not depend on T, on the strips or on the column blocks
@@ -432,8 +433,8 @@ Prepared &prepared() {
 // of n rows takes n + 2 (T-1) turns, and its start is worth one more), a wave
 // being as many warps as the chip holds, or ctas blocks per SM in one wave:
 // fewer and longer strips repeat fewer rows, which is the better choice where
-// short strips would be half repetition (1024^2, T = 4: 9.0 us per step with
-// 3 blocks per SM, 8.4 with 1).  The search takes up to ny turns of the host (three launches
+// short strips would be half repetition (512^2, T = 2: 4.09 us per step with
+// 3 blocks per SM, 3.85 with 2).  The search takes up to ny turns of the host (three launches
 // of 96 x 20000: 95 us of it, now 6.5), so a handle makes it when its shape is set.
 template <int T, bool WALLS>
 cudaError_t strips_t(const VDom &d, int ctas, int *strips) {

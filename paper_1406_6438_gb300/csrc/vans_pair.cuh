@@ -43,7 +43,7 @@ __device__ __forceinline__ f2 sqrt2(f2 x) {
 
 // What a cell's update needs of the porosity, formed once per row and launch:
 // eps, Hc = cs^2 grad eps / eps + g, the drag coefficients and w_i (eps - eps~_i).
-// Fourteen pairs (one spare), seven 16-byte words per lane.
+// Thirteen pairs: six 16-byte words and an 8-byte one per lane.
 struct Por {
     f2 e0, hx, hy, al, be;
     f2 wd[9];              // wd[0] unused
@@ -125,9 +125,12 @@ __device__ __forceinline__ void porosity_terms(const VDom &d, const Row &m, cons
 // 9 (e.u)(e.g) - 3 u.g.  The momentum a cell gains is (1 - omega) j + q = j + V
 // only if ct + omega/2 = 1: near rest j = -V/2 is large (the pressure term
 // p grad eps, which the lattice takes back), so a rounding of 3e-8 in that sum
-// is a spurious force; ct is therefore 1 - omega/2, exact in FP32, and both
-// constants enter unscaled (scaled by 3 and rounded again, the velocity was 2 to
-// 3 times further from 64 bits at tau = 0.55 .. 0.6).
+// is a spurious force; ct is therefore 1 - omega/2, exact in FP32 for omega >= 1
+// (tau <= 1) and off by up to 2^-25 below, and both constants enter unscaled (scaled
+// by 3 and rounded again, the velocity was 2 to 3 times further from 64 bits at
+// tau = 0.55 .. 0.6).  For tau of 1.05 to 8, carrying that rest of ct as well moved the
+// velocity no closer to 64 bits, at rest or flowing, and took 2 % longer: there the
+// error is that of the single-step kinds.
 struct PairMoments {
     f2 dl, R, ux, uy;
 };

@@ -34,23 +34,23 @@ __device__ __forceinline__ void atomic_max_nonneg(float *a, float v) {
 
 // The maxima of a warp into the partial maxima of an emission.
 __device__ __forceinline__ void emit_maxima(const Monitor &mon, int lane, float dmax, float umax, bool bad) {
-            // warp maxima, one atomic per warp
+    // warp maxima, one atomic per warp
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                dmax = fmaxf(dmax, __shfl_xor_sync(VANS_FULL, dmax, off));
-                umax = fmaxf(umax, __shfl_xor_sync(VANS_FULL, umax, off));
-            }
-            bad = __any_sync(VANS_FULL, bad);
-            if (lane == 0) {
-                // one of kMonSlots partial maxima per warp: with every warp on the
-                // same three words the step took 634 us at 4096^2, 420 us spread
-                const int slot = (int)((blockIdx.x * ((blockDim.x * blockDim.y) >> 5) +
-                                        ((threadIdx.y * blockDim.x + threadIdx.x) >> 5)) &
-                                       (kMonSlots - 1));
-                atomic_max_nonneg(&mon.part[slot], bad ? 0.f : dmax);
-                atomic_max_nonneg(&mon.part[kMonSlots + slot], bad ? 0.f : umax);
-                if (bad) atomic_max_nonneg(&mon.part[2 * kMonSlots + slot], 1.f);
-            }
+    for (int off = 16; off > 0; off >>= 1) {
+        dmax = fmaxf(dmax, __shfl_xor_sync(VANS_FULL, dmax, off));
+        umax = fmaxf(umax, __shfl_xor_sync(VANS_FULL, umax, off));
+    }
+    bad = __any_sync(VANS_FULL, bad);
+    if (lane == 0) {
+        // one of kMonSlots partial maxima per warp: with every warp on the
+        // same three words the step took 634 us at 4096^2, 420 us spread
+        const int slot = (int)((blockIdx.x * ((blockDim.x * blockDim.y) >> 5) +
+                                ((threadIdx.y * blockDim.x + threadIdx.x) >> 5)) &
+                               (kMonSlots - 1));
+        atomic_max_nonneg(&mon.part[slot], bad ? 0.f : dmax);
+        atomic_max_nonneg(&mon.part[kMonSlots + slot], bad ? 0.f : umax);
+        if (bad) atomic_max_nonneg(&mon.part[2 * kMonSlots + slot], 1.f);
+    }
 }
 
 // What the update of CPT cells from x0 on in row (y, z) reads: the pulled populations h

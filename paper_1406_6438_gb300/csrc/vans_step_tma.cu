@@ -28,7 +28,7 @@
 //      and by idle lanes: kind 6 takes one cell per thread (64 registers, 24
 //      warps; 160 cells: 76 and 20) in tiles of 64 to 256 cells, rows of one tile without the staged
 //      halo columns: 150 x 110 x 90 58 -> 45 us (floor 34), 250^3 459 -> 392
-//      (360), 90^3 43 -> 25.5, 96 x 64 x 48 14.9 -> 10.9; 256^3 stays with kind 7
+//      (360), 90^3 43 -> 24.6, 96 x 64 x 48 14.9 -> 10.9; 256^3 stays with kind 7
 //      (397 against 414).
 //
 // (Kinds 1 -- a pipeline over contiguous runs of tiles with the porosity rows
@@ -695,7 +695,9 @@ __device__ __forceinline__ void ilv_run(Cur cur, const int *status, int ntiles, 
 // 428 us instead of 411): D3Q19 with one cell per thread fits in 64 registers, so as
 // many blocks as those allow (128^3 63.6 -> 61.1 us, 90^3 26.8 -> 25.5, 96 x 64 x 48
 // 11.3 -> 10.9, 221 x 150 x 150 131.8 -> 130.6), but for 160 cells, where a fifth block
-// costs more than it hides (150 x 110 x 90 44.8 -> 46.3).
+// costs more than it hides (with 2 stages, the faster: 150 x 110 x 90 44.5 -> 45.9,
+// 160^3 110.4 -> 112.8, 140 x 100 x 120 53.7 -> 54.7, 132 x 128 x 64 37.4 -> 38.4,
+// 129 x 60 x 40 12.8 -> 13.6, 155 x 220 x 150 141.4 -> 144.2).
 template <int Q, int NT, bool VEC, bool PL>
 __host__ __device__ constexpr int ilv_blocks() {
     return Q == 19 && !VEC && !PL && NT != 160 ? 65536 / (NT + 32) / 64 : 0;
