@@ -845,7 +845,12 @@ static cudaError_t launch_ring_t(const VDom &d, const float *fin, float *fout, i
     const int per_y = pick_per_y(ncol, d.ny, (long long)sms * occ);
     const long long grid = (long long)ncol * per_y;
     if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    kern<<<(unsigned)grid, nthreads, smem_req, stream>>>(d, fin, fout, ntx, per_y, stages);
+    // kind 2 with more than 2 stages has too few blocks per SM to be bound by DRAM: its
+    // rows' last sectors stored whole cost more than they spare (250 x 128 x 100, 3 stages:
+    // 106 -> 111 us with 4 warps, 113 -> 120 with 8; 2 stages 111 -> 98 and 113 -> 102)
+    VDom dd = d;
+    if (!WS && stages > 2) dd.tails = 0;
+    kern<<<(unsigned)grid, nthreads, smem_req, stream>>>(dd, fin, fout, ntx, per_y, stages);
     return cudaGetLastError();
 }
 
