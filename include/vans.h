@@ -305,8 +305,8 @@ int vans_adjoint_segment(vans_t h, const float *ckpt, float *seg, int len, float
  * as fits the row length, 2 stages): bulk-copy pipeline
  * with a producer warp, persistent CTAs over the row tiles; `warps` compute
  * warps (D2Q9: 2 with cpt 1, or 4 with cpt 1 or 2; D3Q19: 2 to 7 with cpt 1),
- * `rows` = pipeline stages (2..8, D3Q19 with 5 warps ..7, with 6 or 7 ..5: what 227 KB
- * of shared memory hold); ctas must be 0.  VANS_ERR_ARG otherwise. */
+ * `rows` = pipeline stages, as many as 227 KB of shared memory hold: 2..8, but D3Q19 2..7
+ * with 5 warps and 2..5 with 6 or 7; ctas must be 0.  VANS_ERR_ARG otherwise. */
 int vans_set_adjoint_launch(vans_t h, const vans_launch *cfg);
 
 /* Arithmetic of the per-cell reverse step and of the sums of vans_grad_finalize: 32
